@@ -163,7 +163,8 @@ def stencil_step_bytes(n, vec_steps, launches):
 
 
 KERNEL_SOURCES = ("common.cuh", "fft.cuh", "precond.h", "precond_fast.h", "precond_fast.cuh",
-                  "precond_fast_mirror.cu", "precond_fast_circ.cu", "precond.cu")
+                  "precond_fast_mirror.cu", "precond_fast_circ.cu", "precond.cu", "precond_line.h",
+                  "precond_line.cuh", "precond_line.cu")
 
 
 def kernel_sources_sha1():

@@ -18,8 +18,13 @@
 // ||v|| instead of being amplified by the spread of the preconditioner's
 // spectrum.
 //
+// Three sets of kernels: squared operators (p = 2) with nx >= 64 transform along
+// x only and solve along y (precond_line.cuh); the FP32 shifted Laplacian (p = 1,
+// whose B_bar^{-1/2} is no recurrence) uses the register FFTs of
+// precond_fast.cuh from 128 on; everything else the generic kernels below.
+//
 // One preconditioned Lanczos step = 5 kernels:
-//   row-forward (forms v_j, stores it) -> column (fwd * symbol * inv)
+//   row-forward (forms v_j, stores it) -> column (fwd * symbol * inv, or solve)
 //   -> row-mid (inverse rows, g, R g, forward rows) -> column
 //   -> row-last (inverse rows, A v_j, q_j, dot products, alpha/beta, stopping rule).
 #include <cuda_runtime.h>
@@ -33,6 +38,7 @@
 #include "fft.cuh"
 #include "precond.h"
 #include "precond_fast.h"
+#include "precond_line.h"
 #include "trace.h"
 
 namespace gmrf {
@@ -641,10 +647,8 @@ fast::Args fast_args(const PrecondTables& t, const Grid& g, const void* kappa2, 
   a.nx = t.nx;
   a.ny = t.ny;
   a.bc = g.bc;
-  a.power = t.power;
-  a.form = t.form;
   a.kbar2 = (float)t.kbar2;
-  a.roff = t.form == FORM_DIAG ? 0.f : (float)t.kbar2;
+  a.roff = (float)t.kbar2;
   a.dscale = (float)(t.kind == GMRF_PREC_CIRCULANT ? 2.0 / ((double)t.nx * t.ny) : 4.0 / ((double)t.nx * t.ny));
   a.lamx = (const float*)t.lamx;
   a.lamy = (const float*)t.lamy;
@@ -656,10 +660,30 @@ fast::Args fast_args(const PrecondTables& t, const Grid& g, const void* kappa2, 
   a.pairy = (const float4*)t.pairy;
   a.T = (float*)t.S;
   a.tstride = (size_t)t.ny * (t.nx + 2);
-  a.G = (float*)t.G;
   a.Wg = (float*)t.Wg;
   a.kappa2 = (const float*)kappa2;
-  a.kappa2_const = t.form == FORM_DIAG ? 0.f : (float)kc;  // FORM_DIAG without a field: D = 0
+  a.kappa2_const = (float)kc;
+  a.n = g.n;
+  return a;
+}
+
+template <typename R>
+line::Args<R> line_args(const PrecondTables& t, const Grid& g, const void* kappa2, double kc) {
+  line::Args<R> a{};
+  a.nx = t.nx;
+  a.ny = t.ny;
+  a.bc = g.bc;
+  a.form = t.form;
+  a.roff = t.form == FORM_DIAG ? (R)0 : (R)t.kbar2;
+  a.tw = (const typename line::C2<R>::T*)t.ltw;
+  a.pair = (const R*)t.lpair;
+  a.col = (const line::ColCoef<R>*)t.lcol;
+  a.T = (R*)t.S;
+  a.tstride = (size_t)t.ny * (t.nx + 2);
+  a.G = (R*)t.G;
+  a.Wg = (R*)t.Wg;
+  a.kappa2 = (const float*)kappa2;
+  a.kappa2_const = t.form == FORM_DIAG ? (R)0 : (R)kc;  // FORM_DIAG without a field: D = 0
   a.n = g.n;
   return a;
 }
@@ -737,6 +761,21 @@ template <typename R, int KIND>
 cudaError_t run_step(PrecondTables& t, const Grid& g, const void* kappa2, double kc, const LanczosBufs& b,
                      const StepParams& P, cudaStream_t s) {
   if (ensure_ws(t, b.nvec, s)) return cudaErrorMemoryAllocation;
+  if (t.line) {
+    line::Args<R> a = line_args<R>(t, g, kappa2, kc);
+    a.W0 = (R*)b.W[0];
+    a.W1 = (R*)b.W[1];
+    a.V = (R*)b.V;
+    a.P = P;
+    a.st = b.st;
+    a.alpha = b.alpha;
+    a.beta = b.beta;
+    a.alpha_f = b.alpha_f;
+    a.beta2_f = b.beta2_f;
+    a.partials = (Dots<R>*)b.partials;
+    a.counters = b.counters;
+    return KIND == GMRF_PREC_CIRCULANT ? line::step_circ<R>(a, b.nvec, s) : line::step_mirror<R>(a, b.nvec, s);
+  }
   if (t.fast) {
     fast::Args a = fast_args(t, g, kappa2, kc);
     a.W0 = (float*)b.W[0];
@@ -787,6 +826,13 @@ cudaError_t run_apply(PrecondTables& t, const Grid& g, const void* in, void* out
                       void* Sbuf = nullptr) {
   if (!Sbuf && ensure_ws(t, nvec, s)) return cudaErrorMemoryAllocation;
   void* S = Sbuf ? Sbuf : t.S;
+  if (t.line) {
+    line::Args<R> a = line_args<R>(t, g, nullptr, 0.0);
+    a.T = (R*)S;
+    a.in = (const R*)in;
+    a.out = (R*)out;
+    return KIND == GMRF_PREC_CIRCULANT ? line::apply_circ<R>(a, nvec, s) : line::apply_mirror<R>(a, nvec, s);
+  }
   if (t.fast) {
     fast::Args a = fast_args(t, g, nullptr, 0.0);
     a.T = (float*)S;
@@ -808,6 +854,12 @@ template <typename R, int KIND>
 cudaError_t run_operator(PrecondTables& t, const Grid& g, const void* kappa2, double kc, const void* v, void* y,
                          int nvec, cudaStream_t s) {
   if (ensure_ws(t, nvec, s)) return cudaErrorMemoryAllocation;
+  if (t.line) {
+    line::Args<R> a = line_args<R>(t, g, kappa2, kc);
+    a.in = (const R*)v;
+    a.out = (R*)y;
+    return KIND == GMRF_PREC_CIRCULANT ? line::operator_circ<R>(a, nvec, s) : line::operator_mirror<R>(a, nvec, s);
+  }
   if (t.fast) {
     fast::Args a = fast_args(t, g, kappa2, kc);
     a.in = (const float*)v;
@@ -922,6 +974,17 @@ int upload_tables(PrecondTables& t, cudaStream_t s, std::vector<double>& lx64, s
     if (up(&t.pairx, prx.data(), prx.size() * sizeof(R)) || up(&t.pairy, pry.data(), pry.size() * sizeof(R)))
       return -1;
   }
+  line::HostTables lt;
+  std::vector<R> ltw, lpair, lcol;
+  if (t.line) {
+    line::host_tables(t.kind, t.nx, t.ny, t.kbar2, lt);
+    ltw.assign(lt.tw.begin(), lt.tw.end());
+    lpair.assign(lt.pair.begin(), lt.pair.end());
+    lcol.assign(lt.col.begin(), lt.col.end());
+    if (up(&t.ltw, ltw.data(), ltw.size() * sizeof(R)) || up(&t.lpair, lpair.data(), lpair.size() * sizeof(R)) ||
+        up(&t.lcol, lcol.data(), lcol.size() * sizeof(R)))
+      return -1;
+  }
   // host vectors must outlive the async copies
   return cudaStreamSynchronize(s) == cudaSuccess ? 0 : -1;
 }
@@ -945,7 +1008,8 @@ int precond_build(PrecondTables& t, const Grid& g, int kind, int op, double kbar
   t.fp64 = fp64;
   t.kbar2 = kbar2;
   t.bc = g.bc;
-  t.fast = fast_eligible(kind, fp64, g.nx, g.ny);
+  t.line = line_eligible(t.power, g.nx, g.ny);
+  t.fast = fast_eligible(kind, t.power, fp64, g.nx, g.ny);
   int rb = (fp64 ? 2048 : 4096) / g.nx;
   if (rb < 1) rb = 1;
   if (rb > 16) rb = 16;
@@ -991,7 +1055,8 @@ int precond_build(PrecondTables& t, const Grid& g, int kind, int op, double kbar
 }
 
 void precond_free(PrecondTables& t, cudaStream_t s) {
-  void* ps[] = {t.lamx, t.lamy, t.twx, t.twy, t.dctx, t.dcty, t.pairx, t.pairy, t.S, t.G, t.Wg};
+  void* ps[] = {t.lamx, t.lamy, t.twx, t.twy, t.dctx, t.dcty, t.pairx, t.pairy, t.ltw, t.lpair, t.lcol,
+                t.S,    t.G,    t.Wg};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, s);
   t = PrecondTables();
@@ -1000,6 +1065,7 @@ void precond_free(PrecondTables& t, cudaStream_t s) {
 int precond_blocks_per_vector(const PrecondTables& t) {
   if (!t.nx) return 0;
   int nb = t.ny / t.rb;
+  if (t.line) nb = std::max(nb, line_blocks_per_vector(t.nx, t.ny));
   if (t.fast) nb = std::max(nb, t.ny / fast_rows_per_block(t.kind, t.nx));
   return nb;
 }

@@ -51,7 +51,11 @@ struct PrecondTables {
   size_t Wg_bytes = 0;
   int rb = 4;            // rows per row-kernel block (generic path)
   int bc = 0;            // boundary condition of the problem
-  bool fast = false;     // FP32 register-FFT kernels with the transposed spectrum
+  bool fast = false;     // FP32 register-FFT kernels with the transposed spectrum (shifted Laplacian)
+  bool line = false;     // transform along x, recurrence along y (squared operators; precond_line.cuh)
+  void* ltw = nullptr;   // tables of the line kernels (line::HostTables)
+  void* lpair = nullptr;
+  void* lcol = nullptr;
 };
 
 bool precond_size_ok(int64_t n);

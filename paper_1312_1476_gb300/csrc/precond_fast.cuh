@@ -695,24 +695,19 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
 
   // inverse transform of the block's rows
   const float* vsrc = a.in ? a.in + (size_t)s * n : a.V + (slot + (size_t)(j % a.P.nslots)) * n;
-  const float* gsrc = a.form == FORM_CTC ? a.G + (size_t)s * n : vsrc;
   // Rows of 1024 (one per warp, one block per SM at one vector): the arrays
   // the elementwise part reads after the inverse transform are loaded before
   // it, so that their latency overlaps the table staging and the transform
-  // (pa, pb, pc: kappa^2 and v for R_MID; g, v and v_{j-1} for R_LAST).
+  // (pa: kappa^2 for R_MID; pa, pc: v and v_{j-1} for R_LAST).
   constexpr bool PF = LOGL == 9 && G == 1 && (MODE == R_MID || MODE == R_LAST);
-  float2 pa[PF ? E : 1], pb[PF ? E : 1], pc[PF ? E : 1];
+  float2 pa[PF ? E : 1], pc[PF ? E : 1];
   if constexpr (PF) {
     const size_t ro = (size_t)(y0 + tr0) * NX;
     if (MODE == R_MID) {
       load_kap<KIND, E>(a, ro, pa);
-      if (a.form == FORM_CTC) load_row<KIND, E>(pb, vsrc + ro);
     } else {
-      load_row<KIND, E>(pa, gsrc + ro);
-      if (!a.in) {
-        load_row<KIND, E>(pb, vsrc + ro);
-        if (j > 0) load_row<KIND, E>(pc, a.V + (slot + (size_t)((j - 1) % a.P.nslots)) * n + ro);
-      }
+      load_row<KIND, E>(pa, vsrc + ro);
+      if (!a.in && j > 0) load_row<KIND, E>(pc, a.V + (slot + (size_t)((j - 1) % a.P.nslots)) * n + ro);
     }
   }
   stage_tables();
@@ -743,34 +738,12 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
       if (MODE == R_MIDG) load_row<KIND, E>(w, wg + ro);
       const bool hy = MODE == R_MIDG && (y == 0 || y == a.ny - 1);
       const size_t rp = (size_t)((y == 0) ? a.ny - 1 : 0) * NX;
-      // partner row's g (needed for the y-term of R g at this row)
-      float2 gp[E];
-      if (hy && a.form == FORM_CTC) {
-        float wpf = 0.f, wpl = 0.f;
-        float2 wp[E];
-        load_row<KIND, E>(wp, wg + rp);
-        if (ex) {
-          wpl = __shfl_sync(0xffffffffu, wp[E - 1].y, 31);
-          wpf = __shfl_sync(0xffffffffu, wp[0].x, 0);
-        }
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-          const size_t o = rp + pair_off<KIND, E>(lane, i);
-          const float2 kk = a.kappa2 ? *reinterpret_cast<const float2*>(a.kappa2 + o) : f2(a.kappa2_const, a.kappa2_const);
-          const float2 vp = *reinterpret_cast<const float2*>(vsrc + o);
-          float2 t = f2(vp.x + (kk.x - a.roff) * wp[i].x + edge_val<KIND>(a.bc, wp[i].x, w[i].x),
-                        vp.y + (kk.y - a.roff) * wp[i].y + edge_val<KIND>(a.bc, wp[i].y, w[i].y));
-          if (lane == 0 && i == 0) t.x += edge_val<KIND>(a.bc, wp[0].x, wpl);
-          if (lane == 31 && i == E - 1) t.y += edge_val<KIND>(a.bc, wp[E - 1].y, wpf);
-          gp[i] = t;
-        }
-      }
       float wf = 0.f, wl = 0.f;
       if (ex) {
         wl = __shfl_sync(0xffffffffu, w[E - 1].y, 31);
         wf = __shfl_sync(0xffffffffu, w[0].x, 0);
       }
-      // rg = R w (in place), then g = v + rg (squared operator)
+      // R w in place
 #pragma unroll
       for (int i = 0; i < E; ++i) {
         const size_t o = ro + pair_off<KIND, E>(lane, i);
@@ -786,37 +759,7 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
           t.x += edge_val<KIND>(a.bc, w[i].x, wq.x);
           t.y += edge_val<KIND>(a.bc, w[i].y, wq.y);
         }
-        if (a.form == FORM_CTC) {
-          float2 vv;
-          if constexpr (PF) vv = pb[i];
-          else vv = *reinterpret_cast<const float2*>(vsrc + o);
-          t = add2(vv, t);
-        }
         w[i] = t;
-      }
-      if (a.form == FORM_CTC) {
-        store_row<KIND, E>(w, a.G + (size_t)s * n + ro);
-        // r = R g (in place)
-        float gf = 0.f, gl = 0.f;
-        if (ex) {
-          gl = __shfl_sync(0xffffffffu, w[E - 1].y, 31);
-          gf = __shfl_sync(0xffffffffu, w[0].x, 0);
-        }
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-          const size_t o = ro + pair_off<KIND, E>(lane, i);
-          float2 kk;
-          if constexpr (PF) kk = pa[i];
-          else kk = a.kappa2 ? *reinterpret_cast<const float2*>(a.kappa2 + o) : f2(a.kappa2_const, a.kappa2_const);
-          float2 t = f2((kk.x - a.roff) * w[i].x, (kk.y - a.roff) * w[i].y);
-          if (ex && lane == 0 && i == 0) t.x += edge_val<KIND>(a.bc, w[0].x, gl);
-          if (ex && lane == 31 && i == E - 1) t.y += edge_val<KIND>(a.bc, w[E - 1].y, gf);
-          if (hy) {
-            t.x += edge_val<KIND>(a.bc, w[i].x, gp[i].x);
-            t.y += edge_val<KIND>(a.bc, w[i].y, gp[i].y);
-          }
-          w[i] = t;
-        }
       }
     }
     __syncthreads();  // tile rows consumed by every warp before they are rewritten
@@ -825,7 +768,7 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
     tile_store_T<KIND, LOGL>(a, tile, Tv, y0);
     return;
   }
-  // R_LAST: A v = g + h
+  // R_LAST: A v = v + h
   if (a.in) {
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -835,7 +778,7 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
 #pragma unroll
         for (int i = 0; i < E; ++i) gg[i] = pa[i];
       } else {
-        load_row<KIND, E>(gg, gsrc + ro);
+        load_row<KIND, E>(gg, vsrc + ro);
       }
 #pragma unroll
       for (int i = 0; i < E; ++i) gg[i] = add2(gg[i], p[g * E + i]);
@@ -851,22 +794,20 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
 #pragma unroll
   for (int g = 0; g < G; ++g) {
     const size_t ro = (size_t)(y0 + tr0 + g) * NX;
-    float2 gg[E], vv[E], q[E];
+    float2 vv[E], q[E];
     if constexpr (PF) {
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        gg[i] = pa[i];
-        vv[i] = pb[i];
+        vv[i] = pa[i];
         q[i] = pc[i];
       }
     } else {
-      load_row<KIND, E>(gg, gsrc + ro);
       load_row<KIND, E>(vv, vsrc + ro);
       if (j > 0) load_row<KIND, E>(q, Vp + ro);
     }
 #pragma unroll
     for (int i = 0; i < E; ++i) {
-      float2 t = add2(gg[i], p[g * E + i]);
+      float2 t = add2(vv[i], p[g * E + i]);
       if (j > 0) t = f2(t.x - bprev * q[i].x, t.y - bprev * q[i].y);
       q[i] = t;
       d.add_dot2(vv[i].x, t.x);  // Dot2: 10 operations per product instead of 13
@@ -882,10 +823,9 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
 }
 
 // ----------------------------------------------------------------- columns
-// symbol of B_bar^{-p/2} (times the transform normalisation); cx = kappa_bar^2 + lambda_x
+// symbol of B_bar^{-1/2} (times the transform normalisation); cx = kappa_bar^2 + lambda_x
 __device__ __forceinline__ float sym_l(const Args& a, float cx, float lam_y) {
-  const float r = rsqrtf(cx + lam_y);  // lam^{-1/2}; lam^{-1} = r^2 (a few ulp, no division)
-  return (a.power == 2 ? r * r : r) * a.dscale;
+  return rsqrtf(cx + lam_y) * a.dscale;
 }
 __device__ __forceinline__ float sym(const Args& a, float cx, const float* lamy, int ky) {
   return sym_l(a, cx, lamy[ky]);

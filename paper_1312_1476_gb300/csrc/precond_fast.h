@@ -9,10 +9,10 @@
 namespace gmrf {
 namespace fast {
 
-// Arguments of the FP32 register-FFT preconditioner kernels.
+// Arguments of the FP32 register-FFT preconditioner kernels (A = I + P R P
+// with P = B_bar^{-1/2}: the shifted Laplacian).
 struct Args {
-  int nx, ny, bc, power;
-  int form;      // FORM_SHIFT / FORM_CTC / FORM_DIAG (precond.h)
+  int nx, ny, bc;
   float kbar2, dscale;
   float roff;    // R = K - roff
   const float* lamx;
@@ -25,7 +25,6 @@ struct Args {
   const float4* pairy; // mirror columns: 4 planes of ny/4 + 1 float4 (see PrecondTables::pairy)
   float* T;            // transposed spectrum
   size_t tstride;      // floats per vector
-  float* G;            // g = C v (squared operator)
   float* Wg;           // w when the y-boundary terms need a separate pass
   const float* in;
   float* out;
@@ -47,9 +46,10 @@ struct Args {
 
 }  // namespace fast
 
-// The FP32 path with register FFTs covers nx in [128, 2048] and ny in
+// The FP32 path with register FFTs covers the shifted Laplacian (power 1; the
+// squared operators go to precond_line.cuh) with nx in [128, 2048] and ny in
 // [64, 1024] (circulant) or [128, 2048] (mirror), powers of two.
-bool fast_eligible(int kind, bool fp64, int nx, int ny);
+bool fast_eligible(int kind, int power, bool fp64, int nx, int ny);
 int fast_rows_per_block(int kind, int nx);
 
 cudaError_t fast_step_circ(const fast::Args& a, int nvec, cudaStream_t s);

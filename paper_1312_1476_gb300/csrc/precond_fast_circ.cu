@@ -15,9 +15,9 @@ cudaError_t fast_operator_circ(const fast::Args& a, int nvec, cudaStream_t s) {
   return fast::operator_k<GMRF_PREC_CIRCULANT>(a, nvec, s);
 }
 
-bool fast_eligible(int kind, bool fp64, int nx, int ny) {
+bool fast_eligible(int kind, int power, bool fp64, int nx, int ny) {
   auto p2 = [](int v) { return v > 0 && (v & (v - 1)) == 0; };
-  if (fp64 || !p2(nx) || !p2(ny) || nx < 128 || nx > 2048) return false;
+  if (fp64 || power != 1 || !p2(nx) || !p2(ny) || nx < 128 || nx > 2048) return false;
   if (kind == GMRF_PREC_CIRCULANT) return ny >= 64 && ny <= 1024;
   return ny >= 128 && ny <= 2048;
 }
