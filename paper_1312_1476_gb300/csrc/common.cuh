@@ -54,6 +54,17 @@ __device__ __forceinline__ df df_shfl_down(df v, int off) {
 }
 __device__ __forceinline__ double df_to_double(df v) { return (double)v.hi + (double)v.lo; }
 
+__device__ __forceinline__ df sum_add(df a, df b) { return df_add(a, b); }
+__device__ __forceinline__ double sum_add(double a, double b) { return a + b; }
+__device__ __forceinline__ df sum_xor(df v, int m) {
+  return {__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m)};
+}
+__device__ __forceinline__ double sum_xor(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ df sum_from(df v, int lane) {
+  return {__shfl_sync(0xffffffffu, v.hi, lane), __shfl_sync(0xffffffffu, v.lo, lane)};
+}
+__device__ __forceinline__ double sum_from(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
+
 // Accumulator of the three dot products of one Lanczos step:
 //   s1 = v_j . q, s2 = q . q, s3 = v_j . v_j  (all for one vector).
 template <typename T>
@@ -61,6 +72,7 @@ struct Dots;
 
 template <>
 struct Dots<float> {
+  typedef df S;
   df s1, s2, s3;
   __device__ __forceinline__ void zero() { s1 = s2 = s3 = {0.f, 0.f}; }
   __device__ __forceinline__ void add(float v, float q) {
@@ -170,6 +182,7 @@ struct Dot2x2 {
 
 template <>
 struct Dots<double> {
+  typedef double S;
   double s1, s2, s3;
   __device__ __forceinline__ void zero() { s1 = s2 = s3 = 0.0; }
   __device__ __forceinline__ void add(double v, double q) {
@@ -218,6 +231,67 @@ __device__ __forceinline__ A block_reduce(A v, A* scratch) {
   }
   __syncthreads();
   return v;
+}
+
+// The three sums of a Dots over a warp with six additions per lane instead of
+// fifteen: lanes 16-31 take s3, lanes 0-15 s1 and s2 and then lanes 8-15 s2.
+// Returns s1 in lanes 0-7, s2 in 8-15, s3 in 16-31 (all lanes of a range hold the
+// same value).  An FP64 addition occupies the SM's FP64 lanes for 16 cycles per
+// warp, so in the small FP64 steps these additions outweigh the stencil.
+template <typename T>
+__device__ __forceinline__ typename Dots<T>::S warp_sum3(const Dots<T>& v) {
+  typedef typename Dots<T>::S S;
+  const int lane = (threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z)) & 31;
+  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+  S k = h16 ? v.s3 : v.s1;
+  k = sum_add(k, sum_xor(h16 ? v.s1 : v.s3, 16));
+  const S k2 = sum_add(v.s2, sum_xor(v.s2, 16));
+  const S give = (h16 || h8) ? k : k2;
+  if (!h16 && h8) k = k2;
+  k = sum_add(k, sum_xor(give, 8));
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) k = sum_add(k, sum_xor(k, off));
+  return k;
+}
+
+// Sum over the first nw warps of the block, in a fixed order; the result is
+// valid in every lane of warp 0.  Every thread of the block calls it, and a
+// barrier has to come before `scratch` is used again.
+template <typename T>
+__device__ __forceinline__ Dots<T> reduce_warps(const Dots<T>& v, Dots<T>* scratch, int nw) {
+  typedef typename Dots<T>::S S;
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int lane = tid & 31, warp = tid >> 5;
+  S k = warp < nw ? warp_sum3(v) : S();
+  if (nw > 1) {
+    S* sc = reinterpret_cast<S*>(scratch);  // [warp][3]
+    const int f = lane == 0 ? 0 : (lane == 8 ? 1 : 2);
+    if (warp < nw && (lane == 0 || lane == 8 || lane == 16)) sc[warp * 3 + f] = k;
+    __syncthreads();
+    if (warp == 0) {
+      // lane 8 f + i adds the warps i, i + 8, ...
+      const int g = min(lane >> 3, 2), i = lane & 7;
+      k = i < nw ? sc[i * 3 + g] : S();
+      for (int w = i + 8; w < nw; w += 8) k = sum_add(k, sc[w * 3 + g]);
+#pragma unroll
+      for (int off = 4; off > 0; off >>= 1) k = sum_add(k, sum_xor(k, off));
+    }
+  }
+  Dots<T> r;
+  r.s1 = sum_from(k, 0);
+  r.s2 = sum_from(k, 8);
+  r.s3 = sum_from(k, 16);
+  return r;
+}
+template <typename T>
+__device__ __forceinline__ Dots<T> block_sum(const Dots<T>& v, Dots<T>* scratch) {
+  return reduce_warps(v, scratch, (int)(blockDim.x * blockDim.y * blockDim.z) >> 5);
+}
+template <typename T>
+__device__ __forceinline__ Dots<T> block_reduce(const Dots<T>& v, Dots<T>* scratch) {
+  const Dots<T> r = block_sum(v, scratch);
+  __syncthreads();
+  return r;
 }
 
 // ------------------------------------------------------------- iteration state
@@ -288,8 +362,8 @@ __device__ __forceinline__ int sturm_count(const float* __restrict__ af, const f
 
 // Smallest eigenvalue of T_m by multisection over the block's threads on a
 // geometric grid below `hi` (an upper bound).  All threads of the block call
-// it; the result is returned to every thread.  Relative resolution after two
-// rounds with 256+ threads is ~1e-4, ample for the bound's lambda_min^{-1/2}.
+// it; the result is returned to every thread.  Relative resolution 3e-4 or
+// better, whatever the block's size, ample for the bound's lambda_min^{-1/2}.
 __device__ __noinline__ static double smallest_ritz(const float* af, const float* b2f, int m, double hi_in, int* s_int,
                                 float* s_flt) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
@@ -323,7 +397,7 @@ __device__ __noinline__ static double smallest_ritz(const float* af, const float
         nhi = lo * __expf(lr * (float)(t + 1) / (float)nt);
         if (t == nt - 1) nhi = hi;
         nlo = (t == 0) ? lo : lo * __expf(lr * (float)t / (float)nt);
-        again = (round == 0) ? 1 : 0;  // two refinement rounds
+        again = (round == 0 || nhi > nlo * 1.0003f) ? 1 : 0;  // two refinement rounds with 256 threads, three with fewer
       }
       s_flt[0] = nlo;
       s_flt[1] = nhi;
@@ -339,6 +413,58 @@ __device__ __noinline__ static double smallest_ritz(const float* af, const float
   return (double)hi;
 }
 
+// Hands a block's partial sums to the block of vector s that comes last:
+// publish() stores them and counts the block in, one acquire-release operation
+// of thread 0 that orders this record alone (no fence of the whole block, which
+// would wait for every store of q_j), and publish_wait() returns, in every
+// thread, whether the block is the last of the nblk blocks of the vector (the
+// counter is reset by it).  Stores that nobody reads before the kernel ends
+// belong between the two.
+__device__ __forceinline__ unsigned count_in(unsigned* counter) {
+  unsigned t;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
+  return t;
+}
+template <typename T>
+__device__ __forceinline__ unsigned publish(const Dots<T>& d, Dots<T>* partials, unsigned* counter, int s, int blk,
+                                            int nblk) {
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  unsigned t = 0;
+  if (tid == 0) {
+    partials[(size_t)s * nblk + blk] = d;
+    if (nblk > 1) t = count_in(counter + s);
+  }
+  return t;
+}
+__device__ __forceinline__ bool publish_wait(unsigned t, unsigned* counter, int s, int nblk, int* s_flag) {
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  if (tid == 0) {
+    const int last = t == (unsigned)(nblk - 1);  // nblk 1: ticket 0
+    if (last) counter[s] = 0u;
+    *s_flag = last;
+  }
+  __syncthreads();
+  return *s_flag != 0;
+}
+// a record another block published: from L2, whatever an L1 line holds
+__device__ __forceinline__ Dots<float> load_partial(const Dots<float>* p) {
+  const float2* q = reinterpret_cast<const float2*>(p);
+  const float2 a = __ldcg(q), b = __ldcg(q + 1), c = __ldcg(q + 2);
+  Dots<float> d;
+  d.s1 = {a.x, a.y};
+  d.s2 = {b.x, b.y};
+  d.s3 = {c.x, c.y};
+  return d;
+}
+__device__ __forceinline__ Dots<double> load_partial(const Dots<double>* p) {
+  const double* q = reinterpret_cast<const double*>(p);
+  Dots<double> d;
+  d.s1 = __ldcg(q);
+  d.s2 = __ldcg(q + 1);
+  d.s3 = __ldcg(q + 2);
+  return d;
+}
+
 // End of a Lanczos step for vector s, run by the last block of that vector
 // (every thread of the block calls it).  Sums the per-block partial dot
 // products in a fixed order, forms alpha_j and beta_j, advances the LDL^T
@@ -349,6 +475,15 @@ __device__ __noinline__ static double smallest_ritz(const float* af, const float
 // b2_direct >= 0, is b2_direct = ||q_j - alpha_j v_j||^2 summed by a caller
 // that holds both vectors (a second pass; exact also when beta_j << ||q_j||,
 // where the one-pass form cancels to rounding noise).
+//
+// This runs between every two steps, so its latency counts in full.  GB300's
+// dependent FP64 operations take about 64 cycles, a division or square root
+// about 600: the reciprocals 1 / beta_j and 1 / d_j are one division in two
+// lanes of warp 0, and the stopping rule compares squares,
+//   beta_j^2 u^2 / d^2 <= tol^2 (u-energy) theta,
+// so the square roots of the estimate itself are taken only in a step that may
+// stop.  Only as many warps as there are partial sums take part in the sum.
+// Together with warp_sum3: 17.2 -> FILLME.
 template <typename T>
 __device__ static void finish_step(const StepParams& P, int j, int s, const Dots<T>* __restrict__ partials, int nblk,
                             VecState* __restrict__ st, double* __restrict__ alpha, double* __restrict__ beta,
@@ -356,111 +491,102 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
                             int* s_int, float* s_flt, double b2_direct = -1.0) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nt = blockDim.x * blockDim.y * blockDim.z;
-  Dots<T> acc;
-  acc.zero();
-  for (int b = tid; b < nblk; b += nt) acc.merge(partials[(size_t)s * nblk + b]);
-  acc = block_reduce(acc, red_scratch);
+  const int warp = tid >> 5, lane = tid & 31;
+  const int nw = min(nt >> 5, (nblk + 31) >> 5);
   __shared__ int s_need_theta;
   __shared__ double s_theta_hi, s_pfac;
   const size_t mo = (size_t)s * P.m_max;
-  if (tid == 0) {
+  VecState* const v = st + s;
+  Dots<T> acc;
+  acc.zero();
+  if (warp < nw)
+    for (int b = tid; b < nblk; b += 32 * nw) acc.merge(load_partial(partials + (size_t)s * nblk + b));
+  acc = reduce_warps(acc, red_scratch, nw);
+  if (warp == 0) {
     double s1, s2, s3;
-    acc.get(s1, s2, s3);
-    VecState v = st[s];
-    double a = s1;
-    double b2 = b2_direct >= 0.0 ? b2_direct : s2 - 2.0 * a * s1 + a * a * s3;
-    double b = b2 > 0.0 ? sqrt(b2) : 0.0;
-    alpha[mo + j] = a;
-    beta[mo + j] = b;
-    alpha_f[mo + j] = (float)a;
-    beta2_f[mo + j] = (float)(b * b);
-    // LDL^T of T_m: d_0 = a_0, d_j = a_j - b_{j-1}^2 / d_{j-1}; u_0 = 1, u_j = -(b_{j-1}/d_{j-1}) u_{j-1}.
-    // The state keeps 1 / d_{j-1}, so that the step's FP64 chain holds one
-    // division (1 / d_j) and one for 1 / beta_j: GB300's FP64 divisions and
-    // square roots are slow, and this tail runs between every two steps.
-    double d, u;
-    if (j == 0) {
-      d = a;
-      u = 1.0;
-      v.energy = 0.0;
-      v.amax = 0.0;
-      v.bmax = 0.0;
-      v.theta = a;
-    } else {
-      const double r = v.beta_last * v.d_prev;  // b_{j-1} / d_{j-1}
-      d = a - v.beta_last * r;
-      u = -r * v.u_prev;
+    acc.get(s1, s2, s3);  // the same values in every lane
+    const double a = s1;
+    const double b2 = b2_direct >= 0.0 ? b2_direct : s2 - 2.0 * a * s1 + a * a * s3;
+    // LDL^T of T_m: d_0 = a_0, d_j = a_j - b_{j-1}^2 / d_{j-1}; u_0 = 1, u_j = -(b_{j-1}/d_{j-1}) u_{j-1}
+    // (the state keeps 1 / d_{j-1})
+    double d = a, u = 1.0, energy = 0.0, amax = 0.0, bmax = 0.0, theta = a;
+    if (j > 0) {
+      const double r = v->beta_last * v->d_prev;  // b_{j-1} / d_{j-1}
+      d = a - v->beta_last * r;
+      u = -r * v->u_prev;
+      energy = v->energy;
+      amax = v->amax;
+      bmax = v->bmax;
+      theta = v->theta;
     }
-    v.m = j + 1;
-    v.beta_last = b;
-    v.vscale = b > 0.0 ? 1.0 / b : 0.0;
-    v.amax = fmax(v.amax, fabs(a));
-    v.bmax = fmax(v.bmax, b);
-    int need = 0;
-    if (!(isfinite(a) && isfinite(b) && isfinite(d))) {
-      v.status = GMRF_ERR_NUMERIC;
-    } else if (d <= 0.0 || a <= 0.0) {
-      v.status = GMRF_ERR_NOT_SPD;
+    const double b = b2 > 0.0 ? sqrt(b2) : 0.0;
+    const double inv = 1.0 / (lane == 1 ? d : b);
+    const double binv = __shfl_sync(0xffffffffu, inv, 0), dinv = __shfl_sync(0xffffffffu, inv, 1);
+    const bool finite = isfinite(a) && isfinite(b) && isfinite(d);
+    int need = 0, status = VS_RUNNING;
+    double pfac = 0.0, err = 0.0;
+    amax = fmax(amax, fabs(a));
+    bmax = fmax(bmax, b);
+    if (!finite || d <= 0.0 || a <= 0.0) {
+      // the estimate of the last completed step stays on record
+      status = finite ? GMRF_ERR_NOT_SPD : GMRF_ERR_NUMERIC;
+      if (P.solve || j == 0) err = v->err_est;
+      else err = v->beta_last * fabs(v->u_prev) * v->d_prev * rsqrt(energy) * rsqrt(theta);
     } else {
-      const double dinv = 1.0 / d;
-      v.energy += u * u * dinv;
-      v.d_prev = dinv;
-      v.u_prev = u;
-      const double rres = b * fabs(u) * dinv;          // ||r_m|| / ||z||
-      double pfac = rres * rsqrt(v.energy);             // ||r_m|| / ||x_m||
-      if (b <= P.bd_tol * (v.amax + v.bmax)) {
-        v.status = VS_DONE;  // invariant Krylov subspace: x_m is exact
-        v.err_est = 0.0;
-        need = !P.solve;     // theta still wanted for the T_m function of a sample
+      energy += u * u * dinv;
+      const double rres = b * fabs(u) * dinv;  // ||r_m|| / ||z||
+      if (b <= P.bd_tol * (amax + bmax)) {
+        status = VS_DONE;  // invariant Krylov subspace: x_m is exact
+        need = !P.solve;   // theta still wanted for the T_m function of a sample
       } else if (P.solve) {
         // linear solve: x_m = ||z|| V_m T_m^{-1} e_1 is the CG iterate, with
         // relative residual ||r_m|| / ||z|| = beta_m |e_m^T T_m^{-1} e_1|
-        v.err_est = rres;
-        if (rres <= P.tol) v.status = VS_DONE;
-        else if (j + 1 >= P.m_max) v.status = GMRF_ERR_NOT_CONVERGED;
-      } else {
-        double est_lb = pfac * rsqrt(v.theta);  // theta >= theta_min(T_m): a lower bound of est
-        v.err_est = est_lb;
-        if (est_lb <= P.tol || j + 1 >= P.m_max) need = 1;
+        err = rres;
+        if (err <= P.tol) status = VS_DONE;
+        else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
+      } else if (!(rres * rres > P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
+        // est_lb = ||r_m|| / (||x_m|| theta^{1/2}), theta >= theta_min(T_m), is a lower bound of est
+        need = 1;
+        pfac = rres * rsqrt(energy);  // ||r_m|| / ||x_m||
+        err = pfac * rsqrt(theta);
       }
-      s_pfac = pfac;
     }
-    s_need_theta = need;
-    s_theta_hi = v.theta;
-    st[s] = v;
+    if (lane == 0) {
+      alpha[mo + j] = a;
+      beta[mo + j] = b;
+      alpha_f[mo + j] = (float)a;
+      beta2_f[mo + j] = (float)(b * b);
+      if (status == VS_RUNNING || status == VS_DONE || status == GMRF_ERR_NOT_CONVERGED) {
+        v->d_prev = dinv;
+        v->u_prev = u;
+      }
+      v->m = j + 1;
+      v->energy = energy;
+      v->theta = theta;
+      v->err_est = err;
+      v->amax = amax;
+      v->bmax = bmax;
+      v->beta_last = b;
+      v->vscale = b > 0.0 ? binv : 0.0;
+      v->status = status;
+      s_pfac = pfac;
+      s_need_theta = need;
+      s_theta_hi = theta;
+    }
   }
   __syncthreads();
   if (s_need_theta) {
     double th = smallest_ritz(alpha_f + mo, beta2_f + mo, j + 1, s_theta_hi, s_int, s_flt);
     if (tid == 0) {
-      VecState v = st[s];
-      v.theta = th;
-      if (v.status == VS_RUNNING) {
-        double est = s_pfac * rsqrt(th);
-        v.err_est = est;
-        if (est <= P.tol && j + 1 >= v.m_min) v.status = VS_DONE;
-        else if (j + 1 >= P.m_max) v.status = GMRF_ERR_NOT_CONVERGED;
+      v->theta = th;
+      if (v->status == VS_RUNNING) {
+        const double est = s_pfac * rsqrt(th);
+        v->err_est = est;
+        if (est <= P.tol && j + 1 >= v->m_min) v->status = VS_DONE;
+        else if (j + 1 >= P.m_max) v->status = GMRF_ERR_NOT_CONVERGED;
       }
-      st[s] = v;
     }
   }
-}
-
-// Last-block election: returns true in every thread of the block that is the
-// last of the `nblk` blocks of vector s to finish (counter reset by it).
-__device__ __forceinline__ bool last_block(unsigned* counter, int s, int nblk, int* s_flag) {
-  __threadfence();
-  __syncthreads();
-  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  if (tid == 0) {
-    unsigned t = atomicAdd(&counter[s], 1u);
-    int last = (t == (unsigned)(nblk - 1));
-    if (last) counter[s] = 0u;
-    *s_flag = last;
-  }
-  __syncthreads();
-  if (*s_flag) __threadfence();
-  return *s_flag != 0;
 }
 
 // ------------------------------------------------------------------- Philox

@@ -164,10 +164,10 @@ __global__ void __launch_bounds__(NT) k_stencil2d(StencilArgs<T> a) {
     }
   }
   if (!STEP) return;
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x * gridDim.y;
-  if (tid == 0) a.partials[(size_t)s * nblk + blockIdx.x + gridDim.x * blockIdx.y] = d;
-  if (last_block(a.counters, s, nblk, &s_int[3]))
+  const unsigned ticket = publish(d, a.partials, a.counters, s, blockIdx.x + gridDim.x * blockIdx.y, nblk);
+  if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
     finish_step<T>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 
@@ -412,10 +412,11 @@ __global__ void __launch_bounds__(NT3) k_stencil3d(StencilArgs<T> a) {
     }
   }
   if (!STEP) return;
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x * gridDim.y * a.nzc;
-  if (tid == 0) a.partials[(size_t)s * nblk + blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zc)] = d;
-  if (last_block(a.counters, s, nblk, &s_int[3]))
+  const unsigned ticket =
+      publish(d, a.partials, a.counters, s, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * zc), nblk);
+  if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
     finish_step<T>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 

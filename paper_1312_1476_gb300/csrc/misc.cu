@@ -126,14 +126,14 @@ __global__ void k_init(const T* __restrict__ W, size_t n, VecState* st, Dots<T>*
     if constexpr (sizeof(T) == 4) Dots<float>::dot2(d.s3, z[i], z[i]);
     else d.s3 = fma(z[i], z[i], d.s3);
   }
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x;
-  if (threadIdx.x == 0) partials[(size_t)s * nblk + blockIdx.x] = d;
-  if (!last_block(counters, s, nblk, &s_flag)) return;
+  const unsigned ticket = publish(d, partials, counters, s, blockIdx.x, nblk);
+  if (!publish_wait(ticket, counters, s, nblk, &s_flag)) return;
   Dots<T> acc;
   acc.zero();
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) acc.merge(partials[(size_t)s * nblk + b]);
-  acc = block_reduce(acc, red);
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) acc.merge(load_partial(partials + (size_t)s * nblk + b));
+  acc = block_sum(acc, red);
   if (threadIdx.x == 0) {
     double s1, s2, s3;
     acc.get(s1, s2, s3);
@@ -400,7 +400,9 @@ __global__ void k_accumulate(const T* __restrict__ V, int nslots, size_t n, cons
       }
     }
   }
-  if (last_block(counters, s, gridDim.x, &s_flag) && threadIdx.x == 0 && work) acc[s] = a + 1;
+  __syncthreads();  // every thread of the block has read acc[s]
+  const unsigned ticket = threadIdx.x == 0 ? count_in(counters + s) : 0u;
+  if (publish_wait(ticket, counters, s, gridDim.x, &s_flag) && threadIdx.x == 0 && work) acc[s] = a + 1;
 }
 
 // x = sum + compensation (FP32) or the FP64 sum; failures filled as k_assemble does.

@@ -403,10 +403,10 @@ __global__ void __launch_bounds__(256) k_prow(PArgs<R> a) {
       d.add(v, q);
     }
   }
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x;
-  if (tid == 0) a.partials[(size_t)s * nblk + blockIdx.x] = d;
-  if (last_block(a.counters, s, nblk, &s_int[3]))
+  const unsigned ticket = publish(d, a.partials, a.counters, s, blockIdx.x, nblk);
+  if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
     finish_step<R>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 

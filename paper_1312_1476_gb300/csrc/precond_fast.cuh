@@ -815,10 +815,10 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
     }
     store_row<KIND, E>(q, Wo + ro);
   }
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x;
-  if (threadIdx.x == 0) a.partials[(size_t)s * nblk + blockIdx.x] = d;
-  if (last_block(a.counters, s, nblk, &s_int[3]))
+  const unsigned ticket = publish(d, a.partials, a.counters, s, blockIdx.x, nblk);
+  if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
     finish_step<float>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 

@@ -410,9 +410,15 @@ __device__ __forceinline__ void row_forward(const Args<R>& a, const typename C2<
   }
 }
 
-// spectrum row S -> real row pairs p (times L)
+// spectrum row q (load_spectrum) -> real row pairs p (times L)
+template <typename R, int NX>
+__device__ __forceinline__ void load_spectrum(R (&q)[4][4], const R* __restrict__ S, int t) {
+  constexpr int T = line_threads(NX);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) ld4(S + 4 * (t + T * r), q[r]);
+}
 template <typename R, int KIND, int NX>
-__device__ __forceinline__ void row_inverse(const Args<R>& a, typename C2<R>::T (&p)[8], const R* __restrict__ S,
+__device__ __forceinline__ void row_inverse(const Args<R>& a, typename C2<R>::T (&p)[8], const R (&q)[4][4],
                                             const Line<R, NX>& ln, int& ph) {
   typedef typename C2<R>::T C;
   constexpr int L = NX / 2, T = L / 8;
@@ -420,9 +426,6 @@ __device__ __forceinline__ void row_inverse(const Args<R>& a, typename C2<R>::T 
   const int t = ln.t;
   const R h = (R)0.70710678118654752440;
   C v[8], up[4];
-  R q[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) ld4(S + 4 * (t + T * r), q[r]);
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int k = t + T * r;
@@ -507,11 +510,6 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   __shared__ R s_edge[MODE == L_MIDG ? RB : 1][2];
   const int s = blockIdx.y;
   const bool step = a.in == nullptr;
-  int j = 0;
-  if (step) {
-    if (a.st[s].status != VS_RUNNING) return;
-    j = a.st[s].m;
-  }
   Line<R, NX> ln;
   ln.t = threadIdx.x % T;
   ln.id = threadIdx.x / T;
@@ -523,7 +521,21 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   const size_t n = a.n, ro = (size_t)y * NX;
   R* S = a.T + (size_t)s * a.tstride + ro;
   const size_t slot = (size_t)s * a.P.nslots;
-  C p[8];
+  C p[8], pa[8], pb[8], pc[8];
+  // what does not depend on the step index is loaded ahead of the state
+  R q[4][4];
+  if constexpr (MODE != L_FWD && MODE != L_MIDG) load_spectrum<R, NX>(q, S, t);
+  // FP32: so is what the elementwise part reads after the inverse transform
+  // (FP64 has no registers to spare)
+  constexpr bool PF = sizeof(R) == 4;
+  if constexpr (PF && MODE == L_MID) load_kap<R, KIND, T>(a, ro, pa, t);
+  if constexpr (PF && MODE == L_LAST)
+    if (a.form == FORM_CTC) load_row<R, KIND, T>(pa, a.G + (size_t)s * n + ro, t);
+  int j = 0;
+  if (step) {
+    if (a.st[s].status != VS_RUNNING) return;
+    j = a.st[s].m;
+  }
 
   if constexpr (MODE == L_FWD) {
     if (!step) {
@@ -532,12 +544,12 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
       load_row<R, KIND, T>(p, ((j & 1) ? a.W1 : a.W0) + (size_t)s * n + ro, t);
       const R inv_b = (R)a.st[s].vscale;
       if (j > 0) {
-        C q[8];
-        load_row<R, KIND, T>(q, a.V + (slot + (size_t)((j - 1) % a.P.nslots)) * n + ro, t);
+        C o[8];
+        load_row<R, KIND, T>(o, a.V + (slot + (size_t)((j - 1) % a.P.nslots)) * n + ro, t);
         const R coef = (R)a.alpha[(size_t)s * a.P.m_max + (j - 1)];
 #pragma unroll
         for (int r = 0; r < 8; ++r)
-          p[r] = mk<C>((p[r].x - coef * q[r].x) * inv_b, (p[r].y - coef * q[r].y) * inv_b);
+          p[r] = mk<C>((p[r].x - coef * o[r].x) * inv_b, (p[r].y - coef * o[r].y) * inv_b);
       } else {
 #pragma unroll
         for (int r = 0; r < 8; ++r) p[r] = mk<C>(p[r].x * inv_b, p[r].y * inv_b);
@@ -552,17 +564,13 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   }
 
   const R* vsrc = step ? a.V + (slot + (size_t)(j % a.P.nslots)) * n : a.in + (size_t)s * n;
-  const R* gsrc = a.form == FORM_CTC ? a.G + (size_t)s * n : vsrc;
-  // FP32: what the elementwise part reads after the inverse transform is loaded
-  // before it, so that both latencies overlap (FP64 has no registers to spare)
-  constexpr bool PF = sizeof(R) == 4;
-  C pa[8], pb[8], pc[8];
   auto load_mid = [&]() {
-    load_kap<R, KIND, T>(a, ro, pa, t);
+    if (!PF) load_kap<R, KIND, T>(a, ro, pa, t);
     if (a.form == FORM_CTC) load_row<R, KIND, T>(pb, vsrc + ro, t);
   };
   auto load_last = [&]() {
-    load_row<R, KIND, T>(pa, gsrc + ro, t);
+    if (a.form != FORM_CTC) load_row<R, KIND, T>(pa, vsrc + ro, t);
+    else if (!PF) load_row<R, KIND, T>(pa, a.G + (size_t)s * n + ro, t);
     if (step) {
       load_row<R, KIND, T>(pb, vsrc + ro, t);
       if (j > 0) load_row<R, KIND, T>(pc, a.V + (slot + (size_t)((j - 1) % a.P.nslots)) * n + ro, t);
@@ -571,7 +579,7 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   if constexpr (PF && MODE == L_MID) load_mid();
   if constexpr (PF && MODE == L_LAST) load_last();
   if constexpr (MODE == L_MIDG) load_row<R, KIND, T>(p, a.Wg + (size_t)s * n + ro, t);
-  else row_inverse<R, KIND, NX>(a, p, S, ln, ph);
+  else row_inverse<R, KIND, NX>(a, p, q, ln, ph);
   if constexpr (MODE == L_INV) {
     if (live) store_row<R, KIND, T>(p, a.out + (size_t)s * n + ro, t);
     return;
@@ -671,17 +679,17 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
     Dots<R> d;
     d.zero();
     if (live) {
-      store_row<R, KIND, T>(p, ((j & 1) ? a.W0 : a.W1) + (size_t)s * n + ro, t);
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         dot_add(d, pb[r].x, p[r].x);
         dot_add(d, pb[r].y, p[r].y);
       }
     }
-    d = block_reduce(d, red);
+    d = block_sum(d, red);
     const int nblk = gridDim.x;
-    if (threadIdx.x == 0) a.partials[(size_t)s * nblk + blockIdx.x] = d;
-    if (last_block(a.counters, s, nblk, &s_int[3]))
+    const unsigned ticket = publish(d, a.partials, a.counters, s, blockIdx.x, nblk);
+    if (live) store_row<R, KIND, T>(p, ((j & 1) ? a.W0 : a.W1) + (size_t)s * n + ro, t);
+    if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
       finish_step<R>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
   }
 }

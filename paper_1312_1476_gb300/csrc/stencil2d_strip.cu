@@ -363,10 +363,10 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
   cp_async_wait<0>();
   if (!STEP) return;
   if constexpr (sizeof(T) == 4) d = dd.merged();
-  d = block_reduce(d, red);
+  d = block_sum(d, red);
   const int nblk = gridDim.x * gridDim.y;
-  if (threadIdx.x == 0) a.partials[(size_t)s * nblk + blockIdx.x + gridDim.x * blockIdx.y] = d;
-  if (last_block(a.counters, s, nblk, &s_int[3]))
+  const unsigned ticket = publish(d, a.partials, a.counters, s, blockIdx.x + gridDim.x * blockIdx.y, nblk);
+  if (publish_wait(ticket, a.counters, s, nblk, &s_int[3]))
     finish_step<T>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 

@@ -310,9 +310,9 @@ __global__ void __launch_bounds__(NT, kMinBlocks)
       return;
     }
     if (STEP) {
-      const Dots<float> d = block_reduce(dd.merged(), red);
-      if (tid == 0) a.partials[(size_t)s * it.per_vec + li] = d;
-      if (last_block(a.counters, s, it.per_vec, &s_int[3]))
+      const Dots<float> d = block_sum(dd.merged(), red);
+      const unsigned ticket = publish(d, a.partials, a.counters, s, li, it.per_vec);
+      if (publish_wait(ticket, a.counters, s, it.per_vec, &s_int[3]))
         finish_step<float>(a.P, j, s, a.partials, it.per_vec, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red,
                            s_int, s_flt);
     }
