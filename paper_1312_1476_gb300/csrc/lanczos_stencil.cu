@@ -467,8 +467,7 @@ cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s) 
     return cudaGetLastError();
   }
   a.nzc = 1;
-  if (stencil2d_strip_eligible(g, sizeof(T) == 8) &&
-      (STEP || stencil2d_strip_pointers_ok(a.Win, a.Wout, a.kappa2)))
+  if (stencil2d_strip_eligible(g, sizeof(T) == 8))
     return launch_stencil2d_strip<T>(g, a, nvec, STEP, s);
 #define GMRF_L2(OPV, BCV) k_stencil2d<T, OPV, BCV, STEP><<<grd, blk, 0, s>>>(a)
   if (g.op == GMRF_OP_SPDE_SQUARED) {

@@ -5,8 +5,9 @@
 // floats or 2 doubles per lane) and a chunk of rows of one vector, and marches
 // down the rows in slabs of 8 (one row per warp).  Every input row of the
 // strip (q_{j-1}, v_{j-1}, kappa^2) is read once, by 16-byte asynchronous
-// copies (cp.async) issued two slabs ahead into rolling shared-memory rings
-// of 32 rows with a 16-byte x halo on either side; v_j is formed in place of
+// copies (cp.async; single elements where rows are not aligned) issued two slabs
+// ahead into rolling shared-memory rings of 32 rows with a 16-byte x halo on
+// either side; v_j is formed in place of
 // q_{j-1} once a slab's copies have landed.  The squared operators keep a ring of
 // g = B v as well:
 //   shifted   q = B v                  (5-point, needs v rows y-1 .. y+1)
@@ -68,7 +69,7 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid)
   if constexpr (BYTES == 16)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
   else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(d), "l"(src), "n"(BYTES), "r"(n) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -86,18 +87,24 @@ __device__ __forceinline__ void ldk_s(const float* p, float (&o)[VX]) {
   }
 }
 
-template <typename T, int OP, int BC, bool STEP>
+// AL: whole strips (nx a multiple of BX) and 16-byte aligned pointers.  Otherwise
+// rows may start anywhere and the last strip ends inside: the copies move single
+// elements, lane after lane, the rows of v_j and q_j go out the same way from
+// shared memory, and cells outside the grid are kept out of g and of the sums;
+// the arithmetic between is the same.  Measured on 701 x 999, 16 vectors, 5-point,
+// against the tile kernel of lanczos_stencil.cu: 298 -> 61 us a step.
+template <typename T, int OP, int BC, bool STEP, bool AL>
 __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int ychunk) {
   constexpr int VX = strip_vx<T>(), BX = strip_bx<T>(), PW = BX + 2 * VX;
   constexpr bool SQ = OP != GMRF_OP_SHIFTED_LAPLACIAN;
   constexpr int H = SQ ? 2 : 1;
-  // dynamic shared memory (strip_smem_bytes): vr | gr (squared) | vpr (step) | kr;
-  // vr holds q_{j-1} as copied, then v_j; vpr v_{j-1} with the halo columns
+  // dynamic shared memory (strip_smem_bytes): vr | gr (squared) | vpr (step or !AL) | kr;
+  // vr holds q_{j-1} as copied, then v_j; vpr v_{j-1} with the halo columns (!AL: then q_j)
   extern __shared__ __align__(16) unsigned char smraw[];
   T* vr = reinterpret_cast<T*>(smraw);
   T* gr = vr + SR * PW;
   T* vpr = gr + (SQ ? SR * PW : 0);
-  float* kr = reinterpret_cast<float*>(vpr + (STEP ? SR * PW : 0));
+  float* kr = reinterpret_cast<float*>(vpr + (STEP || !AL ? SR * PW : 0));
   __shared__ Dots<T> red[SNT / 32];
   __shared__ int s_int[4];
   __shared__ float s_flt[4];
@@ -146,6 +153,25 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
     }
     const size_t row0 = (size_t)(rin ? gy : 0) * nx;
     const int sl = ring(y);
+    if constexpr (!AL) {
+#pragma unroll
+      for (int part = 0; part <= VX; ++part) {
+        if (part == VX && lane >= 2 * VX) continue;
+        const int col = part < VX ? VX + 32 * part + lane : (lane < VX ? lane : BX + lane);
+        int xx = x0 + col - VX;
+        bool in = rin && xx >= 0 && xx < nx;
+        if (rin && !in && BC == GMRF_BC_PERIODIC) {
+          // only the two columns on either side of the grid are ever read
+          xx = xx < 0 ? xx + nx : xx - nx;
+          in = xx >= 0 && xx < nx;
+        }
+        const size_t i = row0 + (in ? xx : 0);
+        cp_async<sizeof(T)>(vr + sl * PW + col, Win + i, in);
+        if (STEP && j > 0) cp_async<sizeof(T)>(vpr + sl * PW + col, Vp + i, in);
+        if (kfield) cp_async<4>(kr + sl * PW + col, a.kappa2 + i, in);
+      }
+      return;
+    }
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
       if (part == 1 && lane >= 2) continue;
@@ -204,6 +230,9 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
   // test per cell.
   const bool nl = BC == GMRF_BC_NEUMANN && x0 + VX * lane == 0;
   const bool nr = BC == GMRF_BC_NEUMANN && x0 + VX * lane + VX == nx;
+  // the lane's cells inside the grid (!AL)
+  const int nend = nx - (x0 + VX * lane);  // cells from the lane's first one to the end of the row
+  const int nin = min(VX, max(0, nend));
   auto bop_vec = [&](const T* src, int y, const T (&kap)[VX], T (&r)[VX]) {
     const int sl = ring(y), c0 = VX + VX * lane;
     T cc[VX], up[VX], dn[VX];
@@ -230,7 +259,11 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
       for (int e = 0; e < VX; e += 2) {
         const float2 c = make_float2(cc[e], cc[e + 1]);
         const float2 l = make_float2(e == 0 ? lft : cc[e - 1 < 0 ? 0 : e - 1], cc[e]);
-        const float2 rr = make_float2(cc[e + 1], e + 1 == VX - 1 ? rgt : cc[e + 2 < VX ? e + 2 : VX - 1]);
+        float2 rr = make_float2(cc[e + 1], e + 1 == VX - 1 ? rgt : cc[e + 2 < VX ? e + 2 : VX - 1]);
+        if (!AL && BC == GMRF_BC_NEUMANN) {  // the grid may end inside the lane's cells
+          if (nend == e + 1) rr.x = c.x;
+          if (nend == e + 2) rr.y = c.y;
+        }
         float2 t = x2_fma(make_float2(kap[e], kap[e + 1]), c, x2_sub(c, l));
         t = x2_add(t, x2_sub(c, rr));
         t = x2_add(t, x2_sub(c, make_float2(up[e], up[e + 1])));
@@ -242,7 +275,8 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
 #pragma unroll
       for (int e = 0; e < VX; ++e) {
         const T l = e == 0 ? lft : cc[e - 1 < 0 ? 0 : e - 1];
-        const T rr = e == VX - 1 ? rgt : cc[e + 1 < VX ? e + 1 : VX - 1];
+        T rr = e == VX - 1 ? rgt : cc[e + 1 < VX ? e + 1 : VX - 1];
+        if (!AL && BC == GMRF_BC_NEUMANN && nend == e + 1) rr = cc[e];
         T t = kap[e] * cc[e];
         t += cc[e] - l;
         t += cc[e] - rr;
@@ -270,9 +304,11 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
     T kap[VX], gv[VX];
     kap_vec(y, kap);
     bop_vec(vr, y, kap, gv);  // every warp lane takes part (shuffles)
-    if (!rin) {
+    // g is 0 outside the grid (periodic: wrapped values were formed instead)
+    if (!rin || (!AL && BC != GMRF_BC_PERIODIC && nin < VX)) {
 #pragma unroll
-      for (int e = 0; e < VX; ++e) gv[e] = 0;
+      for (int e = 0; e < VX; ++e)
+        if (!rin || e >= nin) gv[e] = 0;
     }
     st16<T, VX>(gr + sl * PW + VX + VX * lane, gv);
     if (lane == 0 || lane == 31) {
@@ -311,15 +347,38 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
 #pragma unroll
       for (int e = 0; e < VX; ++e) q[e] -= bprev * vp[e];
     }
-    const size_t i = (size_t)y * nx + x0 + VX * lane;
-    st16<T, VX>(Wout + i, q);
-    if (STEP) {
-      st16<T, VX>(Vc + i, v);
-      if (a.P.vb) {
-        __nv_bfloat16* pb = vb_at(a.P, s, j, n, i);
-        if (VX == 4) vb_store4(pb, (float)v[0], (float)v[1 % VX], (float)v[2 % VX], (float)v[3 % VX]);
-        else vb_store2(pb, (float)v[0], (float)v[1 % VX]);
+    if constexpr (AL) {
+      const size_t i = (size_t)y * nx + x0 + VX * lane;
+      st16<T, VX>(Wout + i, q);
+      if (STEP) {
+        st16<T, VX>(Vc + i, v);
+        if (a.P.vb) {
+          __nv_bfloat16* pb = vb_at(a.P, s, j, n, i);
+          if (VX == 4) vb_store4(pb, (float)v[0], (float)v[1 % VX], (float)v[2 % VX], (float)v[3 % VX]);
+          else vb_store2(pb, (float)v[0], (float)v[1 % VX]);
+        }
       }
+    } else {
+      // q through v_{j-1}'s row (read above, by this warp alone), then both rows out in order of the columns
+      st16<T, VX>(vpr + sl * PW + c0, q);
+      __syncwarp();
+      const size_t i0 = (size_t)y * nx + x0;
+#pragma unroll
+      for (int e = 0; e < VX; ++e) {
+        const int col = 32 * e + lane;
+        if (x0 + col >= nx) continue;
+        Wout[i0 + col] = vpr[sl * PW + VX + col];
+        if (STEP) {
+          const T vv = vr[sl * PW + VX + col];
+          Vc[i0 + col] = vv;
+          if (a.P.vb) vb_store1(vb_at(a.P, s, j, n, i0 + col), (float)vv);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < VX; ++e)
+        if (e >= nin) q[e] = v[e] = 0;  // no part of the sums
+    }
+    if (STEP) {
       if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int e = 0; e < VX; e += 2) dd.add(make_float2(v[e], v[e + 1]), make_float2(q[e], q[e + 1]));
@@ -370,36 +429,60 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
     finish_step<T>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 
-template <typename T, int OP, bool STEP>
+template <typename T, int OP, bool STEP, bool AL>
 constexpr size_t strip_smem_bytes() {
   constexpr int VX = strip_vx<T>(), BX = strip_bx<T>(), PW = BX + 2 * VX;
   return (size_t)SR * PW * sizeof(T) * (OP != GMRF_OP_SHIFTED_LAPLACIAN ? 2 : 1) +
-         (STEP ? (size_t)SR * PW * sizeof(T) : 0) + (size_t)SR * PW * sizeof(float);
+         (STEP || !AL ? (size_t)SR * PW * sizeof(T) : 0) + (size_t)SR * PW * sizeof(float);
 }
 
+// Rows of a chunk: 64 from 1024 rows on, else 32, halved down to 16 (FP64 5-point:
+// 8) while a vector has fewer than 48 (FP64: 64) blocks.  Smaller chunks shorten a
+// lone vector's step and read the H halo rows of a chunk more often (256 x 256,
+// 13-point, 40 steps, FP32: one vector 782 us with 32 rows, 635 with 16, 595 with 8; 32
+// vectors 1554, 1534, 1757).
 template <typename T>
 int strip_ychunk(const Grid& g) {
-  return g.ny >= 1024 ? 64 : 32;
+  const bool f64 = sizeof(T) == 8;
+  const int strips = (g.nx + strip_bx<T>() - 1) / strip_bx<T>();
+  const int enough = f64 ? 64 : 48, least = f64 && g.op == GMRF_OP_SHIFTED_LAPLACIAN ? 8 : 16;
+  int yc = g.ny >= 1024 ? 64 : 32;
+  while (yc > least && strips * ((g.ny + yc - 1) / yc) < enough) yc /= 2;
+  return yc;
 }
 
-template <typename T, int OP, int BC, bool STEP>
-cudaError_t launch_bc(dim3 grd, const StencilArgs<T>& a, int yc, cudaStream_t s) {
-  constexpr size_t sm = strip_smem_bytes<T, OP, STEP>();
+template <typename T, int OP, int BC, bool STEP, bool AL>
+cudaError_t launch_al(dim3 grd, const StencilArgs<T>& a, int yc, cudaStream_t s) {
+  constexpr size_t sm = strip_smem_bytes<T, OP, STEP, AL>();
   static std::atomic<bool> attr{false};  // several host threads may launch at once
   if (!attr.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(k_stencil2d_strip<T, OP, BC, STEP>,
+    cudaError_t e = cudaFuncSetAttribute(k_stencil2d_strip<T, OP, BC, STEP, AL>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
     attr.store(true, std::memory_order_release);
   }
-  k_stencil2d_strip<T, OP, BC, STEP><<<grd, SNT, sm, s>>>(a, yc);
+  k_stencil2d_strip<T, OP, BC, STEP, AL><<<grd, SNT, sm, s>>>(a, yc);
   return cudaGetLastError();
+}
+
+// 16-byte alignment of the vectors and of the coefficient field
+bool stencil2d_strip_pointers_ok(const void* win, const void* wout, const float* kappa2) {
+  auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+  return al(win) && al(wout) && al(kappa2);
+}
+
+template <typename T, int OP, int BC, bool STEP>
+cudaError_t launch_bc(dim3 grd, const StencilArgs<T>& a, int yc, cudaStream_t s) {
+  const bool al = a.nx % strip_bx<T>() == 0 &&
+                  (STEP ? stencil2d_strip_pointers_ok(a.W0, a.W1, a.kappa2)
+                        : stencil2d_strip_pointers_ok(a.Win, a.Wout, a.kappa2));
+  return al ? launch_al<T, OP, BC, STEP, true>(grd, a, yc, s) : launch_al<T, OP, BC, STEP, false>(grd, a, yc, s);
 }
 
 template <typename T, bool STEP, int OP>
 cudaError_t launch_op(const Grid& g, const StencilArgs<T>& a, int nvec, cudaStream_t s) {
   const int yc = strip_ychunk<T>(g);
-  dim3 grd(g.nx / strip_bx<T>(), (g.ny + yc - 1) / yc, nvec);
+  dim3 grd((g.nx + strip_bx<T>() - 1) / strip_bx<T>(), (g.ny + yc - 1) / yc, nvec);
   switch (g.bc) {
     case GMRF_BC_PERIODIC: return launch_bc<T, OP, GMRF_BC_PERIODIC, STEP>(grd, a, yc, s);
     case GMRF_BC_NEUMANN: return launch_bc<T, OP, GMRF_BC_NEUMANN, STEP>(grd, a, yc, s);
@@ -411,18 +494,14 @@ cudaError_t launch_op(const Grid& g, const StencilArgs<T>& a, int nvec, cudaStre
 
 bool stencil2d_strip_eligible(const Grid& g, bool fp64) {
   const int bx = fp64 ? strip_bx<double>() : strip_bx<float>();
-  return g.dim == 2 && g.nx % bx == 0 && g.ny >= 4 && (int64_t)g.nx * g.ny >= 65536;
+  // half a strip: the tile kernel needs five times as long per cell of its tiles
+  return g.dim == 2 && 2 * g.nx >= bx && g.ny >= 4 && (int64_t)g.nx * g.ny >= 65536;
 }
 
 int stencil2d_strip_blocks_per_vector(const Grid& g, bool fp64) {
   const int bx = fp64 ? strip_bx<double>() : strip_bx<float>();
   const int yc = fp64 ? strip_ychunk<double>(g) : strip_ychunk<float>(g);
-  return (g.nx / bx) * ((g.ny + yc - 1) / yc);
-}
-
-bool stencil2d_strip_pointers_ok(const void* win, const void* wout, const float* kappa2) {
-  auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
-  return al(win) && al(wout) && al(kappa2);
+  return ((g.nx + bx - 1) / bx) * ((g.ny + yc - 1) / yc);
 }
 
 template <typename T>
