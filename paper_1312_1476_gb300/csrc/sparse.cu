@@ -9,10 +9,10 @@
 // solves.  Device side: one thread block per vector, whose working vectors
 // stay in shared memory for a whole Lanczos step:
 //     v_j formed from q_{j-1}, v_{j-1} (as in the lattice steps), stored;
-//     t = F^{-T} v_j     backward substitution, level by level, in place
+//     t = F^{-T} v_j     backward substitution, one merged level after another
 //                        (a group of lanes per row, sized to the rows);
-//     u = Q t            CSR rows, Q read through L2 (shared by all blocks);
-//     u := F^{-1} u      forward substitution, level by level, in place;
+//     Q t                CSR rows, Q read through L2 (shared by all blocks);
+//     u = F^{-1} Q t     forward substitution, likewise;
 //     q_j = u - beta_{j-1} v_{j-1} -> W_out, the three dot products,
 // then alpha_j = v_j . q_j, beta_j = ||q_j - alpha_j v_j|| (a second pass over
 // the vectors in shared memory, exact also where A is close to the identity)
@@ -38,26 +38,15 @@ struct SparseOp {
   int* q_ptr = nullptr;  // Q: [n + 1], [nnz] columns, [nnz] values
   int* q_col = nullptr;
   void* q_val = nullptr;
-  // The two substitutions, each with its rows stored in level order (entry r
-  // of the order is row rows[r]): row pointers [n + 1], columns and values of
-  // the off-diagonal entries, and 1 / F_ii [n], all indexed by r, so a row's
-  // pointers load without going through its row index first.
-  //   forward  (F^{-1}):  the strictly lower part of F by rows
-  //   backward (F^{-T}):  the strictly upper part of F^T by rows (F by columns)
-  int* l_ptr = nullptr;
-  int* l_col = nullptr;
-  void* l_val = nullptr;
-  void* l_dinv = nullptr;
-  int* u_ptr = nullptr;
-  int* u_col = nullptr;
-  void* u_val = nullptr;
-  void* u_dinv = nullptr;
-  int* lev_f = nullptr;     // rows in forward-solve level order [n]
-  int* lev_f_ptr = nullptr; // [nlev_f + 1]
-  int* lev_b = nullptr;     // rows in backward-solve level order [n]
-  int* lev_b_ptr = nullptr; // [nlev_b + 1]
-  int nlev_f = 0, nlev_b = 0;
-  int gs = 1;               // lanes per row in the triangular solves
+  // The two substitutions as schedules of merged levels (TriHost):
+  //   tri[0] forward (F^{-1}), tri[1] backward (F^{-T})
+  struct {
+    int* rec = nullptr;   // [rounds][8] round records
+    int* row = nullptr;   // rows of the rounds
+    int* col = nullptr;   // entries: position in the shared arrays, or -1 (padding)
+    void* val = nullptr;
+    int rounds = 0;
+  } tri[2];
   size_t smem = 0;          // dynamic shared memory of the kernels
 };
 
@@ -232,67 +221,89 @@ struct SpArgs {
   const int* qp;
   const int* qc;
   const T* qv;
-  const int* lp;
-  const int* lc;
-  const T* lv;
-  const T* ldi;
-  const int* up;
-  const int* uc;
-  const T* uv;
-  const T* udi;
-  const int* lf;
-  const int* lfp;
-  int nlf;
-  const int* lb;
-  const int* lbp;
-  int nlb;
+  struct {
+    const int* rec;
+    const int* row;
+    const int* col;
+    const T* val;
+    int rounds;
+  } tri[2];
   int has_f;
-  int gs;  // lanes per row in the triangular solves: a power of two <= 32
 };
 
-// One level-scheduled substitution in place: x_i := (x_i - sum_e val_e x_col_e) * (1 / d_i)
-// for the rows of each level in turn (the reciprocal pivots are stored).  A group of gs lanes (aligned within a
-// warp) takes one row, its lanes striding over the row's entries, and the
-// group sums by shuffles; the block's groups take the level's rows in rounds.
-// The round loop depends only on the level, so every lane of a warp reaches
-// the shuffles (inactive groups add zeros).
+// One substitution by its schedule (TriHost): sm is the block's three arrays
+// of n, side by side; x (the second of them) receives the result.  Round by
+// round, every row of the round is a dot product over positions of sm, a group
+// of lanes per row summed by shuffles, with a barrier after the last round of a
+// merged level.  The records run two rounds ahead and the entries of the next
+// round are loaded before this one's sums and barrier, so the chain of a level
+// holds no global load.
+constexpr int kTriRegs = 8;  // entries of a lane loaded ahead; longer rows read the rest in place
+
 template <typename T>
-__device__ __forceinline__ void tri_solve(const SpArgs<T>& a, const int* __restrict__ rows,
-                                          const int* __restrict__ lptr, int nlev, const int* __restrict__ rp,
-                                          const int* __restrict__ col, const T* __restrict__ val,
-                                          const T* __restrict__ dinv, T* x) {
-  const int gs = a.gs;
-  const int grp = (int)threadIdx.x / gs, sub = (int)threadIdx.x & (gs - 1);
-  const int ngrp = (int)blockDim.x / gs;
-  for (int l = 0; l < nlev; ++l) {
-    const int r0 = __ldg(lptr + l), r1 = __ldg(lptr + l + 1);
-    for (int base = r0; base < r1; base += ngrp) {
-      const int r = base + grp;
-      int i = 0;
-      T acc = 0;
-      if (r < r1) {
-        i = __ldg(rows + r);
-        const int e1 = __ldg(rp + r + 1);
-        for (int e = __ldg(rp + r) + sub; e < e1; e += gs) acc += __ldg(val + e) * x[__ldg(col + e)];
+__device__ __forceinline__ void tri_solve(const SpArgs<T>& a, int dir, const T* sm, T* x) {
+  const int* __restrict__ rec = a.tri[dir].rec;
+  const int* __restrict__ rows = a.tri[dir].row;
+  const int* __restrict__ col = a.tri[dir].col;
+  const T* __restrict__ val = a.tri[dir].val;
+  const int nr = a.tri[dir].rounds;
+  const int tid = (int)threadIdx.x;
+  struct Rec {
+    int4 a, b;  // {entries, slots per lane, lanes, log2 lanes per row}, {rows, row count, last of its level, -}
+  };
+  auto load_rec = [&](int r) -> Rec {
+    const int4* p = reinterpret_cast<const int4*>(rec) + 2 * min(r, nr - 1);
+    return {__ldg(p), __ldg(p + 1)};
+  };
+  int c[kTriRegs];
+  T v[kTriRegs];
+  int row = -1;
+  auto load_entries = [&](const Rec& q) {
+    if (tid >= q.a.z) return;
+    const int grp = tid >> q.a.w;
+    row = grp < q.b.y ? __ldg(rows + q.b.x + grp) : -1;
+#pragma unroll
+    for (int k = 0; k < kTriRegs; ++k) {
+      if (k < q.a.y) {
+        c[k] = __ldg(col + q.a.x + k * q.a.z + tid);
+        v[k] = __ldg(val + q.a.x + k * q.a.z + tid);
       }
-      for (int off = gs >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-      if (r < r1 && sub == 0) x[i] = (x[i] - acc) * __ldg(dinv + r);
     }
-    __syncthreads();
+  };
+  Rec cur = load_rec(0), nxt = load_rec(1);
+  load_entries(cur);
+  for (int r = 0; r < nr; ++r) {
+    const Rec q = cur;
+    const bool on = tid < q.a.z;  // whole warps
+    T s0 = 0, s1 = 0;
+    if (on) {
+#pragma unroll
+      for (int k = 0; k < kTriRegs; ++k)
+        if (k < q.a.y && c[k] >= 0) (k & 1 ? s1 : s0) += v[k] * sm[c[k]];
+      for (int k = kTriRegs; k < q.a.y; ++k) {
+        const int ck = __ldg(col + q.a.x + k * q.a.z + tid);
+        if (ck >= 0) s0 += __ldg(val + q.a.x + k * q.a.z + tid) * sm[ck];
+      }
+    }
+    const int i = row;
+    cur = nxt;
+    nxt = load_rec(r + 2);
+    if (r + 1 < nr) load_entries(cur);
+    if (on) {
+      T acc = s0 + s1;
+      for (int off = (1 << q.a.w) >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+      if (i >= 0 && (tid & ((1 << q.a.w) - 1)) == 0) x[i] = acc;
+    }
+    if (q.b.z) __syncthreads();
   }
 }
 
-// x := F^{-1} x  (forward substitution)
+// F^{-1} (from the third array) and F^{-T} (from the first array), both into
+// the second array
 template <typename T>
-__device__ __forceinline__ void lower_solve(const SpArgs<T>& a, T* x) {
-  tri_solve(a, a.lf, a.lfp, a.nlf, a.lp, a.lc, a.lv, a.ldi, x);
-}
-
-// x := F^{-T} x  (backward substitution)
+__device__ __forceinline__ void lower_solve(const SpArgs<T>& a, T* sm) { tri_solve(a, 0, sm, sm + a.n); }
 template <typename T>
-__device__ __forceinline__ void upper_solve(const SpArgs<T>& a, T* x) {
-  tri_solve(a, a.lb, a.lbp, a.nlb, a.up, a.uc, a.uv, a.udi, x);
-}
+__device__ __forceinline__ void upper_solve(const SpArgs<T>& a, T* sm) { tri_solve(a, 1, sm, sm + a.n); }
 
 // y = Q x for all rows (x, y in shared memory; y written, no barrier)
 template <typename T>
@@ -331,7 +342,7 @@ __global__ void __launch_bounds__(kSpThreads) k_sparse_step(SpArgs<T> a, SpStep<
   const int n = a.n;
   T* sv = reinterpret_cast<T*>(smraw);  // v_j
   T* sw = sv + n;                       // t = F^{-T} v_j
-  T* su = sw + n;                       // u = Q t, then F^{-1} u
+  T* su = sw + n;                       // Q t; F^{-1} Q t goes to sw
   const size_t nn = (size_t)n;
   const T* Win = ((j & 1) ? b.W1 : b.W0) + (size_t)s * nn;
   T* Wout = ((j & 1) ? b.W0 : b.W1) + (size_t)s * nn;
@@ -350,15 +361,15 @@ __global__ void __launch_bounds__(kSpThreads) k_sparse_step(SpArgs<T> a, SpStep<
     const T w = Win[i];
     const T v = j == 0 ? w * inv_b : (w - coef * Vp[i]) * inv_b;
     sv[i] = v;
-    sw[i] = v;
     Vc[i] = v;
   }
   __syncthreads();
   if (a.has_f) {
-    upper_solve(a, sw);
+    upper_solve(a, sv);
     spmv(a, sw, su);
     __syncthreads();
-    lower_solve(a, su);
+    lower_solve(a, sv);
+    su = sw;
   } else {
     spmv(a, sv, su);
     __syncthreads();
@@ -408,20 +419,20 @@ __global__ void __launch_bounds__(kSpThreads) k_sparse_ops(SpArgs<T> a, int mode
   const int n = a.n;
   T* sx = reinterpret_cast<T*>(smraw);
   T* sy = sx + n;
+  T* sz = sy + n;
   const T* x = in + (size_t)blockIdx.x * n;
   T* y = out + (size_t)blockIdx.x * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) sx[i] = x[i];
+  T* src = mode == 3 ? sz : sx;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) src[i] = x[i];
   __syncthreads();
-  T* res = sx;
+  T* res = sy;
   if (mode == 0) {
     spmv(a, sx, sy);
-    res = sy;
   } else if (mode == 1) {
     upper_solve(a, sx);
-    spmv(a, sx, sy);
+    spmv(a, sy, sz);
     __syncthreads();
-    lower_solve(a, sy);
-    res = sy;
+    lower_solve(a, sx);
   } else if (mode == 2) {
     upper_solve(a, sx);
   } else {
@@ -438,22 +449,14 @@ SpArgs<T> sp_args(const SparseOp& S) {
   a.qp = S.q_ptr;
   a.qc = S.q_col;
   a.qv = (const T*)S.q_val;
-  a.lp = S.l_ptr;
-  a.lc = S.l_col;
-  a.lv = (const T*)S.l_val;
-  a.ldi = (const T*)S.l_dinv;
-  a.up = S.u_ptr;
-  a.uc = S.u_col;
-  a.uv = (const T*)S.u_val;
-  a.udi = (const T*)S.u_dinv;
-  a.lf = S.lev_f;
-  a.lfp = S.lev_f_ptr;
-  a.nlf = S.nlev_f;
-  a.lb = S.lev_b;
-  a.lbp = S.lev_b_ptr;
-  a.nlb = S.nlev_b;
+  for (int d = 0; d < 2; ++d) {
+    a.tri[d].rec = S.tri[d].rec;
+    a.tri[d].row = S.tri[d].row;
+    a.tri[d].col = S.tri[d].col;
+    a.tri[d].val = (const T*)S.tri[d].val;
+    a.tri[d].rounds = S.tri[d].rounds;
+  }
   a.has_f = S.has_f ? 1 : 0;
-  a.gs = S.gs;
   return a;
 }
 
@@ -534,6 +537,124 @@ void levels(int n, const std::vector<int>& ptr, const std::vector<int>& col, boo
   rows.assign((size_t)n, 0);
   std::vector<int> fill(lptr.begin(), lptr.end() - 1);
   for (int i = 0; i < n; ++i) rows[(size_t)fill[(size_t)lev[(size_t)i]]++] = i;
+}
+
+// The schedule of one substitution.  Consecutive levels are merged into one:
+// with the rows B of the merged levels and the rows P before them,
+//   x_B = F_BB^{-1} b_B - F_BB^{-1} F_BP x_P,
+// so every row of B is a dot product over right-hand sides of B and results of
+// P, at the price of the fill that the small inverse brings.  A level costs a
+// chain of dependent operations and a barrier whatever it holds (about
+// kLevelCycles), an entry its share of the FP64 lanes and of the loads (kEntryCycles),
+// so the next level is merged while the entries it adds cost less than that.
+// Merged rows stay below kMergedRow entries.  The values are formed in FP64.
+// kEntryCycles and the six entries per lane are the best of a sweep on the
+// Figure 3 matrix, 256 samples, drop tolerance 1e-3 / 1e-5 / 1e-2 (FP64): 4.2 /
+// 6.4 / 12.5 ms a call at 3 cycles, 6.4 / 6.4 / 14.4 at 1.5, 7.9 / 7.3 / 19.4 at 14;
+// 10.7 / 29.1 / 26.3 ms level by level.  The factor with 1e-3 goes from 204 to 39
+// levels and from 13.4k to 29.5k entries.
+struct TriHost {
+  std::vector<int> rec, row, col;
+  std::vector<double> val;
+};
+constexpr double kLevelCycles = 500.0;
+constexpr double kEntryCycles = 3.0;
+constexpr int kMergedRow = 128;
+
+// rows in level order (lptr); ptr/col/val the off-diagonal entries of each row;
+// b and x the positions of the right-hand side and of the result in the shared arrays
+void tri_schedule(int n, const std::vector<int>& rows, const std::vector<int>& lptr, const std::vector<int>& ptr,
+                  const std::vector<int>& col, const std::vector<double>& val, const std::vector<double>& dg, int b0,
+                  int x0, TriHost& out) {
+  const int nlev = (int)lptr.size() - 1;
+  typedef std::vector<std::pair<int, double>> Expr;  // (position, coefficient), ascending
+  std::vector<Expr> expr((size_t)n);  // of the rows of the merged level being built
+  std::vector<int> in_block((size_t)n, -1);
+  std::vector<double> acc((size_t)std::max(b0, x0) + n, 0.0);
+  std::vector<int> stamp(acc.size(), -1), used;
+  int block = 0, mark = 0;
+  auto row_expr = [&](int i, Expr& e) {
+    ++mark;
+    used.clear();
+    auto add = [&](int at, double w) {
+      if (stamp[(size_t)at] != mark) {
+        stamp[(size_t)at] = mark;
+        acc[(size_t)at] = 0.0;
+        used.push_back(at);
+      }
+      acc[(size_t)at] += w;
+    };
+    add(b0 + i, 1.0);
+    for (int q = ptr[(size_t)i]; q < ptr[(size_t)i + 1]; ++q) {
+      const int k = col[(size_t)q];
+      if (in_block[(size_t)k] == block)
+        for (const auto& t : expr[(size_t)k]) add(t.first, -val[(size_t)q] * t.second);
+      else
+        add(x0 + k, -val[(size_t)q]);
+    }
+    std::sort(used.begin(), used.end());
+    e.clear();
+    for (int at : used) e.emplace_back(at, acc[(size_t)at] / dg[(size_t)i]);
+  };
+  out = TriHost();
+  std::vector<Expr> cand;
+  for (int l = 0; l < nlev;) {
+    ++block;
+    std::vector<int> members;
+    int end = l;
+    for (; end < nlev; ++end) {
+      cand.clear();
+      double extra = 0.0;
+      size_t longest = 0;
+      for (int q = lptr[(size_t)end]; q < lptr[(size_t)end + 1]; ++q) {
+        const int i = rows[(size_t)q];
+        Expr e;
+        row_expr(i, e);
+        extra += (double)e.size() - (double)(ptr[(size_t)i + 1] - ptr[(size_t)i] + 1);
+        longest = std::max(longest, e.size());
+        cand.push_back(std::move(e));
+      }
+      if (end > l && (extra * kEntryCycles > kLevelCycles || longest > (size_t)kMergedRow)) break;
+      for (int q = lptr[(size_t)end]; q < lptr[(size_t)end + 1]; ++q) {
+        const int i = rows[(size_t)q];
+        expr[(size_t)i] = std::move(cand[(size_t)(q - lptr[(size_t)end])]);
+        in_block[(size_t)i] = block;
+        members.push_back(i);
+      }
+    }
+    l = end;
+    // rounds of the merged level: rows by length, about six entries per lane
+    std::stable_sort(members.begin(), members.end(),
+                     [&](int p, int q) { return expr[(size_t)p].size() > expr[(size_t)q].size(); });
+    double mean = 0.0;
+    for (int i : members) mean += (double)expr[(size_t)i].size();
+    mean /= (double)members.size();
+    int lg = 0;
+    while (lg < 5 && 6.0 * (1 << lg) < mean) ++lg;
+    const int per = kSpThreads >> lg;
+    for (size_t m0 = 0; m0 < members.size(); m0 += (size_t)per) {
+      const int cnt = (int)std::min((size_t)per, members.size() - m0);
+      const int lanes = ((cnt << lg) + 31) / 32 * 32;
+      const int slots = (int)((expr[(size_t)members[m0]].size() + (1u << lg) - 1) >> lg);
+      const size_t off = out.col.size();
+      const int rec[8] = {(int)off, slots, lanes, lg, (int)out.row.size(), cnt,
+                          m0 + (size_t)per >= members.size() ? 1 : 0, 0};
+      out.rec.insert(out.rec.end(), rec, rec + 8);
+      out.col.resize(off + (size_t)slots * lanes, -1);
+      out.val.resize(out.col.size(), 0.0);
+      for (int r = 0; r < cnt; ++r) {
+        const int i = members[m0 + (size_t)r];
+        out.row.push_back(i);
+        const Expr& e = expr[(size_t)i];
+        for (size_t t = 0; t < e.size(); ++t) {
+          const size_t at = off + (t >> lg) * (size_t)lanes + ((size_t)r << lg) + (t & ((1u << lg) - 1));
+          out.col[at] = e[t].first;
+          out.val[at] = e[t].second;
+        }
+      }
+    }
+    for (int i : members) Expr().swap(expr[(size_t)i]);
+  }
 }
 
 template <typename T>
@@ -628,53 +749,21 @@ int sparse_create(SparseOp** out, const gmrf_sparse_desc* d, bool fp64, cudaStre
     std::vector<int> rf, pf, rb, pb;
     levels(n, lp, lc, true, rf, pf);
     levels(n, up, uc, false, rb, pb);
-    S->nlev_f = (int)pf.size() - 1;
-    S->nlev_b = (int)pb.size() - 1;
-    // lanes per row: the power of two at or above the mean off-diagonal row length (1 .. 32)
-    const double mean_row = (double)lc.size() / (double)n;
-    while (S->gs < 32 && S->gs < mean_row) S->gs *= 2;
-    // rows in level order: pointers, entries and 1 / F_ii indexed by the position r
-    auto by_level = [&](const std::vector<int>& rows, const std::vector<int>& ptr, const std::vector<int>& col,
-                        const std::vector<double>& val, std::vector<int>& optr, std::vector<int>& ocol,
-                        std::vector<double>& oval, std::vector<double>& odinv) {
-      optr.assign((size_t)n + 1, 0);
-      ocol.clear();
-      oval.clear();
-      odinv.assign((size_t)n, 0.0);
-      for (int q = 0; q < n; ++q) {
-        const int i = rows[(size_t)q];
-        for (int e = ptr[(size_t)i]; e < ptr[(size_t)i + 1]; ++e) {
-          ocol.push_back(col[(size_t)e]);
-          oval.push_back(val[(size_t)e]);
-        }
-        optr[(size_t)q + 1] = (int)ocol.size();
-        odinv[(size_t)q] = 1.0 / dg[(size_t)i];
-      }
-    };
-    std::vector<int> lp2, lc2, up2, uc2;
-    std::vector<double> lv2, ld2, uv2, ud2;
-    by_level(rf, lp, lc, lv, lp2, lc2, lv2, ld2);
-    by_level(rb, up, uc, uv, up2, uc2, uv2, ud2);
-    r = upload_i(&S->l_ptr, lp2, s);
-    if (r == GMRF_OK) r = upload_i(&S->l_col, lc2, s);
-    if (r == GMRF_OK) r = upload_i(&S->u_ptr, up2, s);
-    if (r == GMRF_OK) r = upload_i(&S->u_col, uc2, s);
-    if (r == GMRF_OK) r = upload_i(&S->lev_f, rf, s);
-    if (r == GMRF_OK) r = upload_i(&S->lev_f_ptr, pf, s);
-    if (r == GMRF_OK) r = upload_i(&S->lev_b, rb, s);
-    if (r == GMRF_OK) r = upload_i(&S->lev_b_ptr, pb, s);
-    if (r == GMRF_OK) {
-      if (fp64) {
-        r = upload<double>(&S->l_val, lv2, s);
-        if (r == GMRF_OK) r = upload<double>(&S->u_val, uv2, s);
-        if (r == GMRF_OK) r = upload<double>(&S->l_dinv, ld2, s);
-        if (r == GMRF_OK) r = upload<double>(&S->u_dinv, ud2, s);
-      } else {
-        r = upload<float>(&S->l_val, lv2, s);
-        if (r == GMRF_OK) r = upload<float>(&S->u_val, uv2, s);
-        if (r == GMRF_OK) r = upload<float>(&S->l_dinv, ld2, s);
-        if (r == GMRF_OK) r = upload<float>(&S->u_dinv, ud2, s);
-      }
+    // shared arrays of the kernels: 0 .. n - 1 the input of F^{-T}, n .. 2n - 1 the results, 2n .. 3n - 1 the input of F^{-1}
+    TriHost th[2];
+    try {
+      tri_schedule(n, rf, pf, lp, lc, lv, dg, 2 * n, n, th[0]);
+      tri_schedule(n, rb, pb, up, uc, uv, dg, 0, n, th[1]);
+    } catch (const std::bad_alloc&) {
+      return fail(GMRF_ERR_OOM);
+    }
+    for (int d = 0; d < 2 && r == GMRF_OK; ++d) {
+      S->tri[d].rounds = (int)th[d].rec.size() / 8;
+      r = upload_i(&S->tri[d].rec, th[d].rec, s);
+      if (r == GMRF_OK) r = upload_i(&S->tri[d].row, th[d].row, s);
+      if (r == GMRF_OK) r = upload_i(&S->tri[d].col, th[d].col, s);
+      if (r == GMRF_OK)
+        r = fp64 ? upload<double>(&S->tri[d].val, th[d].val, s) : upload<float>(&S->tri[d].val, th[d].val, s);
     }
   }
   if (r != GMRF_OK) {
@@ -688,8 +777,8 @@ int sparse_create(SparseOp** out, const gmrf_sparse_desc* d, bool fp64, cudaStre
 
 void sparse_free(SparseOp* S, cudaStream_t s) {
   if (!S) return;
-  void* ps[] = {S->q_ptr, S->q_col, S->q_val, S->l_ptr,  S->l_col,  S->l_val,     S->l_dinv,    S->u_ptr,
-                S->u_col, S->u_val, S->u_dinv, S->lev_f, S->lev_f_ptr, S->lev_b, S->lev_b_ptr};
+  void* ps[] = {S->q_ptr,      S->q_col,      S->q_val,      S->tri[0].rec, S->tri[0].row, S->tri[0].col,
+                S->tri[0].val, S->tri[1].rec, S->tri[1].row, S->tri[1].col, S->tri[1].val};
   for (void* p : ps)
     if (p) cudaFreeAsync(p, s);
   cudaGetLastError();
