@@ -17,9 +17,10 @@
 //   shifted:  B v = kappa^2 v + L v            (5-point 2-D, 7-point 3-D)
 //   squared:  Q v = B (B v)                    (13-point 2-D, two passes in smem)
 // 2-D: 32x16 tiles with a halo of 1 (shifted) or 2 (squared) in shared memory.
-// 3-D: 32x8 tiles in x-y marching over a chunk of z planes with the inputs of
-// later planes prefetched; the centre column is kept in registers, the plane
-// with its x-y halo in a double-buffered shared tile.
+// 3-D: stencil3d_tma.cu and stencil3d_flat.cu; wider than the latter takes, 32x8
+// tiles in x-y marching over a chunk of z planes with the inputs of later planes
+// prefetched; the centre column is kept in registers, the plane with its x-y halo
+// in a double-buffered shared tile.
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -184,7 +185,7 @@ constexpr int NT3 = TX * TY3;
 template <typename T, int VX>
 struct Raw {
   T w[VX], vp[VX];
-  float k[VX];
+  T k[VX];  // a constant kappa^2 keeps its FP64 value
 };
 
 template <typename T, int VX>
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(NT3) k_stencil3d(StencilArgs<T> a) {
 #pragma unroll
     for (int e = 0; e < VX; ++e) {
       r.w[e] = r.vp[e] = (T)0;
-      r.k[e] = 0.f;
+      r.k[e] = (T)0;
     }
     int zz = gz, yy = gy;
     bool in = own && gz >= 0 && gz < nz;
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(NT3) k_stencil3d(StencilArgs<T> a) {
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < VX; ++e) r.k[e] = (float)a.kappa2_const;
+      for (int e = 0; e < VX; ++e) r.k[e] = a.kappa2_const;
     }
   };
   // halo ring cells of this thread
@@ -446,6 +447,7 @@ cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s) 
           (STEP || stencil3d_tma_pointers_ok(a.Win, a.Wout, a.kappa2)))
         return launch_stencil3d_tma(g, a, nvec, STEP, s);
     }
+    if (stencil3d_flat_eligible(g)) return launch_stencil3d_flat<T>(g, a, nvec, STEP, s);
     const int vx = vx3(g, sizeof(T) == 8);
     a.nzc = nz_chunks(g, vx);
     blk = dim3(TX, TY3);
@@ -510,7 +512,9 @@ StencilArgs<T> make_args(const Grid& g, const void* kappa2, double kc) {
 int stencil_blocks_per_vector(const Grid& g) {
   if (g.dim == 3) {
     // the widest tile (VX = 1) has the most blocks; the TMA kernel's items
-    const int r = ((g.nx + TX - 1) / TX) * ((g.ny + TY3 - 1) / TY3) * nz_chunks(g, 1);
+    const int r = stencil3d_flat_eligible(g)
+                      ? stencil3d_flat_blocks_per_vector(g)
+                      : ((g.nx + TX - 1) / TX) * ((g.ny + TY3 - 1) / TY3) * nz_chunks(g, 1);
     const int t = stencil3d_tma_eligible(g, false) ? stencil3d_tma_items_per_vector(g) : 0;
     return r > t ? r : t;
   }
