@@ -951,10 +951,9 @@ int gmrf_sample(gmrf_problem* p, const gmrf_sample_opts* o, void* x_out, gmrf_re
         CKR(ensure(p->work, (size_t)c * n * es, p->ws));
         CK(traced(KC_ASSEMBLE, s, 1, [&] { return assemble(1.0, p->work.p); }));
         CK(traced(KC_PRE_APPLY, s, 3, [&] {
-          return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, c, s);
+          return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, c, s,
+                                      1.0 / std::sqrt(p->tau));
         }));
-        CK(traced(KC_OTHER, s, 1,
-                  [&] { return launch_scale(p->fp64, xdst, (size_t)c * n, 1.0 / std::sqrt(p->tau), s); }));
       }
       // accuracy check: the direct residual r = z - A u_cg
       CKR(check_vectors(p, c, p->zre.p, p->ucg.p, b.st, p->st_host, o->tol, est.data(), s));
@@ -1059,8 +1058,8 @@ int gmrf_solve(gmrf_problem* p, const gmrf_solve_opts* o, const void* b_in, void
       CK(traced(KC_ASSEMBLE, s, 1,
                 [&] { return launch_assemble(p->fp64, n, b, (double*)p->y.p, m_max, 1.0, p->work.p, s); }));
       CK(traced(KC_PRE_APPLY, s, 3,
-                [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, c, s); }));
-      CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, xdst, (size_t)c * n, 1.0 / p->tau, s); }));
+                [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, c, s,
+                                                   1.0 / p->tau); }));
     }
     if (!x_dev)
       CK(cudaMemcpyAsync((char*)x_out + (size_t)s0 * n * es, xdst, (size_t)c * n * es, cudaMemcpyDeviceToHost, s));
@@ -1239,10 +1238,9 @@ int gmrf_sample_logdet(gmrf_problem* p, const gmrf_sample_opts* so, const gmrf_l
           return launch_assemble_dual(p->fp64, n, bs, (double*)p->y.p, m_max, 1.0, p->work.p, ycg, p->ucg.p, s);
         }));
         CK(traced(KC_PRE_APPLY, s, 3, [&] {
-          return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, nsc, s);
+          return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, xdst, nsc, s,
+                                      1.0 / std::sqrt(p->tau));
         }));
-        CK(traced(KC_OTHER, s, 1,
-                  [&] { return launch_scale(p->fp64, xdst, (size_t)nsc * n, 1.0 / std::sqrt(p->tau), s); }));
       }
       // accuracy check of the samples, with the same resumption as gmrf_sample
       CKR(check_vectors(p, nsc, p->zre.p, p->ucg.p, b.st, p->st_host, so->tol, est.data(), s));
@@ -1307,17 +1305,16 @@ int gmrf_apply(gmrf_problem* p, int32_t which, int64_t nvec, const void* v, void
     }
   } else if (which == 0) {
     CK(traced(KC_STENCIL_STEP, s, 1, [&] {
-      return launch_stencil_apply(p->g, p->fp64, p->kappa2.p, p->kappa2_const, vin, yout, (int)nvec, s);
+      return launch_stencil_apply(p->g, p->fp64, p->kappa2.p, p->kappa2_const, vin, yout, (int)nvec, s, p->tau);
     }));
-    CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, yout, (size_t)nvec * n, p->tau, s); }));
   } else if (which == 1) {
     CK(traced(KC_PRE_APPLY, s, 5, [&] {
       return launch_precond_operator(p->pre, p->g, p->fp64, p->kappa2.p, p->kappa2_const, vin, yout, (int)nvec, s);
     }));
   } else {
     CK(traced(KC_PRE_APPLY, s, 3,
-              [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, vin, yout, (int)nvec, s); }));
-    CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, yout, (size_t)nvec * n, 1.0 / std::sqrt(p->tau), s); }));
+              [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, vin, yout, (int)nvec, s,
+                                                 1.0 / std::sqrt(p->tau)); }));
   }
   if (!yd) CK(cudaMemcpyAsync(y, yout, bytes, cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
@@ -1524,9 +1521,8 @@ extern "C" int gmrf_apply_inv_sqrt_noalloc(gmrf_problem* p, int64_t nvec, const 
   // the spectrum is fully written by the forward row pass before it is read:
   // nothing in the shared scratch has to start at zero
   CK(traced(KC_PRE_APPLY, s, 3, [&] {
-    return launch_precond_apply_with(p->pre, p->g, p->fp64, v, y, (int)nvec, scratch, s);
+    return launch_precond_apply_with(p->pre, p->g, p->fp64, v, y, (int)nvec, scratch, s, 1.0 / std::sqrt(p->tau));
   }));
-  CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, y, (size_t)nvec * p->g.n, 1.0 / std::sqrt(p->tau), s); }));
   CK(cudaStreamSynchronize(s));
   trace_collect();
   CKR(leave(p));

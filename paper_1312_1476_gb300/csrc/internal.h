@@ -61,7 +61,7 @@ cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, do
                                 const LanczosBufs& b, const StepParams& P, cudaStream_t s);
 // y = Q v for nvec vectors (no Lanczos bookkeeping).
 cudaError_t launch_stencil_apply(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
-                                 const void* v, void* y, int nvec, cudaStream_t s);
+                                 const void* v, void* y, int nvec, cudaStream_t s, double scale = 1.0);
 
 // stencil3d_tma.cu -------------------------------------------------------------
 // The TMA-staged 3-D 7-point step / apply serves FP32 grids with Dirichlet or

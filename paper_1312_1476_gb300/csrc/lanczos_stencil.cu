@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(NT) k_stencil2d(StencilArgs<T> a) {
     else qv = bop2<T, BC, VW>(vs, tx + H, ty + H, gx, gy, nx, ny, kap);
     if (OP == GMRF_OP_SPDE_PLUS_DIAG && a.kappa2) qv += (T)__ldg(a.kappa2 + i) * vs[(ty + H) * VW + tx + H];
     if (!STEP) {
-      Wout[i] = qv;
+      Wout[i] = qv * a.scale;
     } else {
       const T v = vs[(ty + H) * VW + tx + H];
       T q = qv;
@@ -387,6 +387,10 @@ __global__ void __launch_bounds__(NT3) k_stencil3d(StencilArgs<T> a) {
         qo[e] = r;
         if (STEP) d.add(vc[e], r);
       }
+      if (!STEP) {
+#pragma unroll
+        for (int e = 0; e < VX; ++e) qo[e] *= a.scale;
+      }
       vstore<T, VX>(Wout + i, qo);
       if (STEP) {
         vstore<T, VX>(Vc + i, vc);
@@ -549,16 +553,18 @@ cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, do
 }
 
 cudaError_t launch_stencil_apply(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
-                                 const void* v, void* y, int nvec, cudaStream_t s) {
+                                 const void* v, void* y, int nvec, cudaStream_t s, double scale) {
   if (fp64) {
     auto a = make_args<double>(g, kappa2, kappa2_const);
     a.Win = (const double*)v;
     a.Wout = (double*)y;
+    a.scale = scale;
     return dispatch<double, false>(g, a, nvec, s);
   }
   auto a = make_args<float>(g, kappa2, kappa2_const);
   a.Win = (const float*)v;
   a.Wout = (float*)y;
+  a.scale = (float)scale;
   return dispatch<float, false>(g, a, nvec, s);
 }
 

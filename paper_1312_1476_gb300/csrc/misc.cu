@@ -695,6 +695,7 @@ cudaError_t launch_loop_cond(cudaGraphConditionalHandle h, const VecState* st, i
 }
 
 cudaError_t launch_scale(bool fp64, void* x, size_t count, double a, cudaStream_t s) {
+  if (a == 1.0) return cudaSuccess;
   const int grid = grid_for(count, 256);
   if (fp64) k_scale<double><<<grid, 256, 0, s>>>((double*)x, count, a);
   else k_scale<float><<<grid, 256, 0, s>>>((float*)x, count, (float)a);

@@ -823,7 +823,7 @@ cudaError_t run_step(PrecondTables& t, const Grid& g, const void* kappa2, double
 // Sbuf: spectrum workspace (nullptr = the tables' own, grown on demand)
 template <typename R, int KIND>
 cudaError_t run_apply(PrecondTables& t, const Grid& g, const void* in, void* out, int nvec, cudaStream_t s,
-                      void* Sbuf = nullptr) {
+                      double scale, void* Sbuf = nullptr) {
   if (!Sbuf && ensure_ws(t, nvec, s)) return cudaErrorMemoryAllocation;
   void* S = Sbuf ? Sbuf : t.S;
   if (t.line) {
@@ -831,14 +831,24 @@ cudaError_t run_apply(PrecondTables& t, const Grid& g, const void* in, void* out
     a.T = (R*)S;
     a.in = (const R*)in;
     a.out = (R*)out;
+    a.scale = (R)scale;
     return KIND == GMRF_PREC_CIRCULANT ? line::apply_circ<R>(a, nvec, s) : line::apply_mirror<R>(a, nvec, s);
   }
+  // the other kernels leave the factor to a pass of its own
+  auto scaled = [&]() -> cudaError_t {
+    if (scale == 1.0) return cudaSuccess;
+    trace_begin(KC_OTHER, s);
+    const cudaError_t e = launch_scale(sizeof(R) == 8, out, (size_t)nvec * g.n, scale, s);
+    trace_end(KC_OTHER, s);
+    return e;
+  };
   if (t.fast) {
     fast::Args a = fast_args(t, g, nullptr, 0.0);
     a.T = (float*)S;
     a.in = (const float*)in;
     a.out = (float*)out;
-    return KIND == GMRF_PREC_CIRCULANT ? fast_apply_circ(a, nvec, s) : fast_apply_mirror(a, nvec, s);
+    CKE((KIND == GMRF_PREC_CIRCULANT ? fast_apply_circ(a, nvec, s) : fast_apply_mirror(a, nvec, s)));
+    return scaled();
   }
   PArgs<R> a = base_args<R>(t, g, nullptr, 0.0);
   a.S = (R*)S;
@@ -847,7 +857,7 @@ cudaError_t run_apply(PrecondTables& t, const Grid& g, const void* in, void* out
   CKE((row_launch<R, KIND, M_FWD_PLAIN>(t, a, nvec, s, KC_PRE_APPLY)));
   CKE((col_launch<R, KIND>(t, a, nvec, 0, s, KC_PRE_APPLY)));
   CKE((row_launch<R, KIND, M_INV_PLAIN>(t, a, nvec, s, KC_PRE_APPLY)));
-  return cudaSuccess;
+  return scaled();
 }
 
 template <typename R, int KIND>
@@ -1097,14 +1107,14 @@ cudaError_t launch_precond_step(PrecondTables& t, const Grid& g, bool fp64, cons
 }
 
 cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int which, const void* in, void* out,
-                                 int nvec, cudaStream_t s) {
+                                 int nvec, cudaStream_t s, double scale) {
   (void)which;
   if (fp64) {
-    if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<double, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s);
-    return run_apply<double, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s);
+    if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<double, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, scale);
+    return run_apply<double, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, scale);
   }
-  if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<float, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s);
-  return run_apply<float, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s);
+  if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<float, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, scale);
+  return run_apply<float, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, scale);
 }
 
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec) {
@@ -1112,14 +1122,14 @@ size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec) {
 }
 
 cudaError_t launch_precond_apply_with(PrecondTables& t, const Grid& g, bool fp64, const void* in, void* out, int nvec,
-                                      void* S, cudaStream_t s) {
+                                      void* S, cudaStream_t s, double scale) {
   if (!S) return cudaErrorInvalidValue;
   if (fp64) {
-    if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<double, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, S);
-    return run_apply<double, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, S);
+    if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<double, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, scale, S);
+    return run_apply<double, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, scale, S);
   }
-  if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<float, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, S);
-  return run_apply<float, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, S);
+  if (t.kind == GMRF_PREC_CIRCULANT) return run_apply<float, GMRF_PREC_CIRCULANT>(t, g, in, out, nvec, s, scale, S);
+  return run_apply<float, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, scale, S);
 }
 
 cudaError_t launch_precond_operator(PrecondTables& t, const Grid& g, bool fp64, const void* kappa2,

@@ -72,15 +72,15 @@ size_t precond_extra_bytes(const PrecondTables& t, size_t es);
 // I + P R P for the shifted one, R = B - B_bar).
 cudaError_t launch_precond_step(PrecondTables& t, const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
                                 const LanczosBufs& b, const StepParams& P, cudaStream_t s);
-// out = B_bar^{-p/2} in for nvec vectors (tau not applied).
+// out = scale B_bar^{-p/2} in for nvec vectors (tau not applied).
 cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int which, const void* in, void* out,
-                                 int nvec, cudaStream_t s);
+                                 int nvec, cudaStream_t s, double scale = 1.0);
 // Same as launch_precond_apply, but the spectrum lives in the caller's
 // workspace S of at least precond_apply_scratch_bytes(t, nvec) bytes; no
 // device memory is allocated.
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec);
 cudaError_t launch_precond_apply_with(PrecondTables& t, const Grid& g, bool fp64, const void* in, void* out, int nvec,
-                                      void* S, cudaStream_t s);
+                                      void* S, cudaStream_t s, double scale = 1.0);
 // y = A v for nvec vectors.
 cudaError_t launch_precond_operator(PrecondTables& t, const Grid& g, bool fp64, const void* kappa2,
                                     double kappa2_const, const void* v, void* y, int nvec, cudaStream_t s);

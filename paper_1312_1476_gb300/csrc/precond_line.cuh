@@ -581,6 +581,8 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   if constexpr (MODE == L_MIDG) load_row<R, KIND, T>(p, a.Wg + (size_t)s * n + ro, t);
   else row_inverse<R, KIND, NX>(a, p, q, ln, ph);
   if constexpr (MODE == L_INV) {
+#pragma unroll
+    for (int r = 0; r < 8; ++r) p[r] = mk<C>(p[r].x * a.scale, p[r].y * a.scale);
     if (live) store_row<R, KIND, T>(p, a.out + (size_t)s * n + ro, t);
     return;
   }
@@ -920,7 +922,7 @@ cudaError_t step_k(const Args<R>& a, int nvec, cudaStream_t s) {
   return row_launch<R, KIND, L_LAST>(a, nvec, s, KC_PRE_ROW_LAST);
 }
 
-// out = B_bar^{-1} in
+// out = scale B_bar^{-1} in
 template <typename R, int KIND>
 cudaError_t apply_k(const Args<R>& a, int nvec, cudaStream_t s) {
   LINE_CK((row_launch<R, KIND, L_FWD>(a, nvec, s, KC_PRE_APPLY)));

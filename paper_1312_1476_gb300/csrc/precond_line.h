@@ -48,6 +48,7 @@ struct Args {
   R* Wg;                // w when the y-boundary terms need a separate pass
   const R* in;
   R* out;
+  R scale;              // of out (L_INV)
   const float* kappa2;
   R kappa2_const;
   size_t n;

@@ -140,12 +140,14 @@ int finish_samples(gmrf_server* sv, int a, int k, Req& r) {
     CKR(ensure(p->work, (size_t)k * n * es, p->ws));
     CK(traced(KC_ASSEMBLE, s, 1,
               [&] { return launch_assemble_dual(p->fp64, n, bs, y, m_max, 1.0, p->work.p, ycg, p->ucg.p, s); }));
-    if (p->sp)
+    if (p->sp) {
       CK(traced(KC_PRE_APPLY, s, 1, [&] { return launch_sparse_ops(*p->sp, 2, p->work.p, dst, k, s); }));
-    else
-      CK(traced(KC_PRE_APPLY, s, 3,
-                [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, dst, k, s); }));
-    CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, dst, (size_t)k * n, xs, s); }));
+      CK(traced(KC_OTHER, s, 1, [&] { return launch_scale(p->fp64, dst, (size_t)k * n, xs, s); }));
+    } else {
+      CK(traced(KC_PRE_APPLY, s, 3, [&] {
+        return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, p->work.p, dst, k, s, xs);
+      }));
+    }
   } else {
     CK(traced(KC_ASSEMBLE, s, 1,
               [&] { return launch_assemble_dual(p->fp64, n, bs, y, m_max, xs, dst, ycg, p->ucg.p, s); }));

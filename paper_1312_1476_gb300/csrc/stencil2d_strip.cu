@@ -347,6 +347,10 @@ __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int y
 #pragma unroll
       for (int e = 0; e < VX; ++e) q[e] -= bprev * vp[e];
     }
+    if (!STEP) {
+#pragma unroll
+      for (int e = 0; e < VX; ++e) q[e] *= a.scale;
+    }
     if constexpr (AL) {
       const size_t i = (size_t)y * nx + x0 + VX * lane;
       st16<T, VX>(Wout + i, q);

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(FNT, 3) k_stencil3d_flat(StencilArgs<T> a, int
         res[e] = (T)0;  // no part of the sums
         continue;
       }
-      Wout[o + FNT * e] = res[e];
+      Wout[o + FNT * e] = STEP ? res[e] : res[e] * a.scale;
       if (STEP) {
         Vc[o + FNT * e] = vc[e];
         if (a.P.vb) vb_store1(vb_at(a.P, s, j, n, o + FNT * e), (float)vc[e]);

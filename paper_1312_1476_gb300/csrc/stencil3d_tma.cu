@@ -257,6 +257,10 @@ __global__ void __launch_bounds__(NT, kMinBlocks)
             dd.add(make_float2(vc[2], vc[3]), make_float2(qo[2], qo[3]));
           }
           const size_t i = (size_t)gx + (size_t)nx * gy + plane * z;
+          if (!STEP) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) qo[e] *= a.scale;
+          }
           *reinterpret_cast<float4*>(Wout + i) = make_float4(qo[0], qo[1], qo[2], qo[3]);
           if (STEP) {
             *reinterpret_cast<float4*>(Vc + i) = make_float4(vc[0], vc[1], vc[2], vc[3]);
@@ -284,6 +288,10 @@ __global__ void __launch_bounds__(NT, kMinBlocks)
             dd.add(make_float2(vc[2], vc[3]), make_float2(qo[2], qo[3]));
           }
           const size_t i = (size_t)gx + (size_t)nx * gy + plane * z;
+          if (!STEP) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) qo[e] *= a.scale;
+          }
           *reinterpret_cast<float4*>(Wout + i) = make_float4(qo[0], qo[1], qo[2], qo[3]);
           if (STEP) {
             *reinterpret_cast<float4*>(Vc + i) = make_float4(vc[0], vc[1], vc[2], vc[3]);

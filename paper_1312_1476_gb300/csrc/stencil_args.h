@@ -12,7 +12,8 @@ namespace gmrf {
 template <typename T>
 struct StencilArgs {
   const T* Win;  // apply mode: v
-  T* Wout;       // apply mode: y
+  T* Wout;       // apply mode: y = scale Q v
+  T scale;
   T* W0;         // step mode: q ping-pong, W[j & 1] read, W[(j+1) & 1] written
   T* W1;
   T* V;  // basis ring base
