@@ -16,7 +16,7 @@
 // which keeps the FP32 rounding relative to the result for smooth v):
 //   shifted:  B v = kappa^2 v + L v            (5-point 2-D, 7-point 3-D)
 //   squared:  Q v = B (B v)                    (13-point 2-D, two passes in smem)
-// 2-D: 32x16 tiles with a halo of 1 (shifted) or 2 (squared) in shared memory.
+// 2-D: 32x16 (FP64 32x8) tiles with a halo of 1 (shifted) or 2 (squared) in shared memory.
 // 3-D: stencil3d_tma.cu and stencil3d_flat.cu; wider than the latter takes, 32x8
 // tiles in x-y marching over a chunk of z planes with the inputs of later planes
 // prefetched; the centre column is kept in registers, the plane with its x-y halo
@@ -30,8 +30,15 @@ namespace gmrf {
 namespace {
 
 constexpr int TX = 32;
-constexpr int TY = 16;
-constexpr int NT = TX * TY;
+// Rows of a 2-D tile, two of them a thread's: half the additions of a sum over
+// the block, and half its barriers, per cell.  FP64 tiles are 8 rows, so that a
+// small grid spreads over more SMs (their FP64 lanes bound it), FP32 tiles 16.
+// 64 x 64 periodic, about 26 steps, one vector and 256, 16 rows and one a thread
+// (512 threads) before: FP64 636 -> 588 us and 3119 -> 2732, FP32 514 -> 508 and
+// 1872 -> 1549.
+constexpr int CPT = 2;
+template <typename T>
+__host__ __device__ constexpr int tile_y() { return sizeof(T) == 8 ? 8 : 16; }
 
 __device__ __forceinline__ int wrapi(int g, int n) {
   g %= n;
@@ -61,7 +68,8 @@ __device__ __forceinline__ T bop2(const T* a, int cx, int cy, int gx, int gy, in
 // SPDE_PLUS_DIAG: Q v = B(B v) + D v with B = kappa_c^2 I + L (constant
 // coefficient, kappa2_const) and D = diag(kappa2 field, or 0).
 template <typename T, int OP, int BC, bool STEP>
-__global__ void __launch_bounds__(NT) k_stencil2d(StencilArgs<T> a) {
+__global__ void __launch_bounds__(TX * tile_y<T>() / CPT) k_stencil2d(StencilArgs<T> a) {
+  constexpr int TY = tile_y<T>(), NT = TX * TY / CPT;
   constexpr bool SQ = OP != GMRF_OP_SHIFTED_LAPLACIAN;  // B applied twice
   constexpr int H = SQ ? 2 : 1;
   constexpr int VW = TX + 2 * H, VH = TY + 2 * H;
@@ -141,21 +149,23 @@ __global__ void __launch_bounds__(NT) k_stencil2d(StencilArgs<T> a) {
     }
     __syncthreads();
   }
-  const int gx = x0 + tx, gy = y0 + ty;
-  const bool own = gx < nx && gy < ny;
   Dots<T> d;
   d.zero();
-  if (own) {
+#pragma unroll
+  for (int c = 0; c < CPT; ++c) {
+    const int cy = ty + c * (TY / CPT);
+    const int gx = x0 + tx, gy = y0 + cy;
+    if (gx >= nx || gy >= ny) continue;
     const size_t i = (size_t)gx + (size_t)nx * gy;
     const T kap = OP == GMRF_OP_SPDE_PLUS_DIAG ? a.kappa2_const : kap_at<T>(a.kappa2, a.kappa2_const, i);
     T qv;
-    if (SQ) qv = bop2<T, BC, GW>(gs, tx + 1, ty + 1, gx, gy, nx, ny, kap);
-    else qv = bop2<T, BC, VW>(vs, tx + H, ty + H, gx, gy, nx, ny, kap);
-    if (OP == GMRF_OP_SPDE_PLUS_DIAG && a.kappa2) qv += (T)__ldg(a.kappa2 + i) * vs[(ty + H) * VW + tx + H];
+    if (SQ) qv = bop2<T, BC, GW>(gs, tx + 1, cy + 1, gx, gy, nx, ny, kap);
+    else qv = bop2<T, BC, VW>(vs, tx + H, cy + H, gx, gy, nx, ny, kap);
+    if (OP == GMRF_OP_SPDE_PLUS_DIAG && a.kappa2) qv += (T)__ldg(a.kappa2 + i) * vs[(cy + H) * VW + tx + H];
     if (!STEP) {
       Wout[i] = qv * a.scale;
     } else {
-      const T v = vs[(ty + H) * VW + tx + H];
+      const T v = vs[(cy + H) * VW + tx + H];
       T q = qv;
       if (j > 0) q -= bprev * Vp[i];
       Wout[i] = q;
@@ -442,7 +452,8 @@ int nz_chunks(const Grid& g, int vx) {
 
 template <typename T, bool STEP>
 cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s) {
-  dim3 blk(TX, TY);
+  constexpr int TY = tile_y<T>();
+  dim3 blk(TX, TY / CPT);
   dim3 grd((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, nvec);
   if (g.dim == 3) {
     if (g.op != GMRF_OP_SHIFTED_LAPLACIAN) return cudaErrorNotSupported;
@@ -522,7 +533,7 @@ int stencil_blocks_per_vector(const Grid& g) {
     const int t = stencil3d_tma_eligible(g, false) ? stencil3d_tma_items_per_vector(g) : 0;
     return r > t ? r : t;
   }
-  int r = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
+  int r = ((g.nx + TX - 1) / TX) * ((g.ny + tile_y<double>() - 1) / tile_y<double>());
   for (int fp64 = 0; fp64 < 2; ++fp64)
     if (stencil2d_strip_eligible(g, fp64 != 0)) r = std::max(r, stencil2d_strip_blocks_per_vector(g, fp64 != 0));
   return r;
