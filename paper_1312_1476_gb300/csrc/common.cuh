@@ -308,7 +308,7 @@ struct VecState {
   double theta;   // smallest Ritz value theta_min (upper estimate)
   double err_est; // relative Theorem 1 estimate at m
   double amax;    // max |alpha_i|
-  double bmax;    // max beta_i
+  double bmax;    // max beta_i, i < m - 1
   double beta_last;  // beta_{m-1}
   double vscale;     // 1 / ||z|| at m = 0, then 1 / beta_{m-1}: the scale of v_m (one division per step)
 };
@@ -465,6 +465,11 @@ __device__ __forceinline__ Dots<double> load_partial(const Dots<double>* p) {
   return d;
 }
 
+// beta_j^2 from the three sums, or the caller's
+__device__ __forceinline__ double step_b2(double a, double s2, double s3, double b2_direct) {
+  return b2_direct >= 0.0 ? b2_direct : s2 - 2.0 * a * a + a * a * s3;
+}
+
 // End of a Lanczos step for vector s, run by the last block of that vector
 // (every thread of the block calls it).  Sums the per-block partial dot
 // products in a fixed order, forms alpha_j and beta_j, advances the LDL^T
@@ -478,12 +483,17 @@ __device__ __forceinline__ Dots<double> load_partial(const Dots<double>* p) {
 //
 // This runs between every two steps, so its latency counts in full.  GB300's
 // dependent FP64 operations take about 64 cycles, a division or square root
-// about 600: the reciprocals 1 / beta_j and 1 / d_j are one division in two
-// lanes of warp 0, and the stopping rule compares squares,
+// about 600: what the next step needs (alpha, beta, 1 / beta) is one warp's
+// reciprocal square root, the recurrence of T_m (1 / d_j) and the stopping rule,
 //   beta_j^2 u^2 / d^2 <= tol^2 (u-energy) theta,
-// so the square roots of the estimate itself are taken only in a step that may
-// stop.  Only as many warps as there are partial sums take part in the sum.
-// Together with warp_sum3: 17.2 -> FILLME.
+// another's, both from beta_j^2; square roots of the estimate are taken only in a
+// step that may stop.  The state's fields are loaded ahead, one per lane, and
+// written one by one: a copy of the record costs the kernels this is inlined into
+// registers (spills in the 3-D step's item loop, 330 -> 344 us at 256^3, 8 vectors).
+// Only as many warps as there are partial sums take part in the sum.
+// With warp_sum3 and publish(), before and now: FP64 64 x 64 step 17.2 -> 11.7 us
+// (one vector; 12.7 with all of it in one warp), 93 -> 48 us (256 vectors); 512 x 512
+// row-last pass, 320 vectors, 346 -> 317 us.
 template <typename T>
 __device__ static void finish_step(const StepParams& P, int j, int s, const Dots<T>* __restrict__ partials, int nblk,
                             VecState* __restrict__ st, double* __restrict__ alpha, double* __restrict__ beta,
@@ -497,66 +507,90 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
   __shared__ double s_theta_hi, s_pfac;
   const size_t mo = (size_t)s * P.m_max;
   VecState* const v = st + s;
+  // the state's fields d_prev .. beta_last, one per lane of warp 1 (the only warp
+  // of a block of 32 threads: warp 0), in flight while the sums are formed
+  const int wb = nt > 32 ? 1 : 0;
+  const double field = warp == wb && lane < 8 ? (&v->d_prev)[lane] : 0.0;
+  __shared__ double s_sum[3];
   Dots<T> acc;
   acc.zero();
   if (warp < nw)
     for (int b = tid; b < nblk; b += 32 * nw) acc.merge(load_partial(partials + (size_t)s * nblk + b));
   acc = reduce_warps(acc, red_scratch, nw);
+  if (tid == 0) acc.get(s_sum[0], s_sum[1], s_sum[2]);
+  __syncthreads();
+  const double a = s_sum[0];
+  // warp 0: alpha_j, beta_j and 1 / beta_j, which the next step waits for
   if (warp == 0) {
-    double s1, s2, s3;
-    acc.get(s1, s2, s3);  // the same values in every lane
-    const double a = s1;
-    const double b2 = b2_direct >= 0.0 ? b2_direct : s2 - 2.0 * a * s1 + a * a * s3;
-    // LDL^T of T_m: d_0 = a_0, d_j = a_j - b_{j-1}^2 / d_{j-1}; u_0 = 1, u_j = -(b_{j-1}/d_{j-1}) u_{j-1}
-    // (the state keeps 1 / d_{j-1})
-    double d = a, u = 1.0, energy = 0.0, amax = 0.0, bmax = 0.0, theta = a;
-    if (j > 0) {
-      const double r = v->beta_last * v->d_prev;  // b_{j-1} / d_{j-1}
-      d = a - v->beta_last * r;
-      u = -r * v->u_prev;
-      energy = v->energy;
-      amax = v->amax;
-      bmax = v->bmax;
-      theta = v->theta;
-    }
-    const double b = b2 > 0.0 ? sqrt(b2) : 0.0;
-    const double inv = 1.0 / (lane == 1 ? d : b);
-    const double binv = __shfl_sync(0xffffffffu, inv, 0), dinv = __shfl_sync(0xffffffffu, inv, 1);
-    const bool finite = isfinite(a) && isfinite(b) && isfinite(d);
-    int need = 0, status = VS_RUNNING;
-    double pfac = 0.0, err = 0.0;
-    amax = fmax(amax, fabs(a));
-    bmax = fmax(bmax, b);
-    if (!finite || d <= 0.0 || a <= 0.0) {
-      // the estimate of the last completed step stays on record
-      status = finite ? GMRF_ERR_NOT_SPD : GMRF_ERR_NUMERIC;
-      if (P.solve || j == 0) err = v->err_est;
-      else err = v->beta_last * fabs(v->u_prev) * v->d_prev * rsqrt(energy) * rsqrt(theta);
-    } else {
-      energy += u * u * dinv;
-      const double rres = b * fabs(u) * dinv;  // ||r_m|| / ||z||
-      if (b <= P.bd_tol * (amax + bmax)) {
-        status = VS_DONE;  // invariant Krylov subspace: x_m is exact
-        need = !P.solve;   // theta still wanted for the T_m function of a sample
-      } else if (P.solve) {
-        // linear solve: x_m = ||z|| V_m T_m^{-1} e_1 is the CG iterate, with
-        // relative residual ||r_m|| / ||z|| = beta_m |e_m^T T_m^{-1} e_1|
-        err = rres;
-        if (err <= P.tol) status = VS_DONE;
-        else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
-      } else if (!(rres * rres > P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
-        // est_lb = ||r_m|| / (||x_m|| theta^{1/2}), theta >= theta_min(T_m), is a lower bound of est
-        need = 1;
-        pfac = rres * rsqrt(energy);  // ||r_m|| / ||x_m||
-        err = pfac * rsqrt(theta);
-      }
-    }
+    const double b2 = step_b2(a, s_sum[1], s_sum[2], b2_direct);
+    const double y = b2 > 0.0 ? rsqrt(b2) : 0.0;
+    // beta_j = sqrt(b2) from y by one Newton step on the residual b2 - b^2
+    double b = b2 * y;
+    b = fma(fma(-b, b, b2), 0.5 * y, b);
+    if (!(b2 < 1e300) || b2 < 1e-290) b = b2 > 0.0 ? sqrt(b2) : 0.0;  // where b2 or y leave the range (or are no numbers)
     if (lane == 0) {
       alpha[mo + j] = a;
       beta[mo + j] = b;
       alpha_f[mo + j] = (float)a;
       beta2_f[mo + j] = (float)(b * b);
-      if (status == VS_RUNNING || status == VS_DONE || status == GMRF_ERR_NOT_CONVERGED) {
+      v->beta_last = b;
+      v->vscale = y;
+    }
+  }
+  // warp 1: the recurrence of T_m and the stopping rule, on beta_j^2
+  if (warp == wb) {
+    const double b2 = step_b2(a, s_sum[1], s_sum[2], b2_direct);
+    auto prev = [&](int k) { return __shfl_sync(0xffffffffu, field, k); };
+    const double d_prev = prev(0), u_prev = prev(1), b_prev = prev(7);
+    // LDL^T of T_m: d_0 = a_0, d_j = a_j - b_{j-1}^2 / d_{j-1}; u_0 = 1, u_j = -(b_{j-1}/d_{j-1}) u_{j-1}
+    // (the state keeps 1 / d_{j-1})
+    double d = a, u = 1.0, energy = prev(2), theta = prev(3), err = prev(4), amax = prev(5), bmax = prev(6);
+    if (j > 0) {
+      const double r = b_prev * d_prev;  // b_{j-1} / d_{j-1}
+      d = a - b_prev * r;
+      u = -r * u_prev;
+    } else {
+      energy = amax = bmax = 0.0;
+      theta = a;
+    }
+    const double dinv = 1.0 / d;
+    const bool finite = isfinite(a) && isfinite(b2) && isfinite(d);
+    int need = 0, status = VS_RUNNING;
+    double pfac = 0.0;
+    amax = fmax(amax, fabs(a));
+    if (j > 0) bmax = fmax(bmax, b_prev);
+    if (!finite || d <= 0.0 || a <= 0.0) {
+      // the estimate of the last completed step stays on record
+      status = finite ? GMRF_ERR_NOT_SPD : GMRF_ERR_NUMERIC;
+      if (j > 0) {
+        err = b_prev * fabs(u_prev) * d_prev;
+        if (!P.solve) err *= rsqrt(energy) * rsqrt(theta);
+      }
+    } else {
+      const double ud = u * dinv;
+      energy += u * ud;
+      const double rr2 = fmax(b2, 0.0) * (ud * ud);  // (||r_m|| / ||z||)^2
+      const double bd = P.bd_tol * (amax + bmax);
+      if (b2 <= bd * bd) {
+        status = VS_DONE;  // invariant Krylov subspace: x_m is exact
+        err = 0.0;
+        need = !P.solve;   // theta still wanted for the T_m function of a sample
+      } else if (P.solve) {
+        // linear solve: x_m = ||z|| V_m T_m^{-1} e_1 is the CG iterate, with
+        // relative residual ||r_m|| / ||z|| = beta_m |e_m^T T_m^{-1} e_1|
+        const bool done = rr2 <= P.tol * P.tol;
+        if (done) status = VS_DONE;
+        else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
+        if (status != VS_RUNNING) err = sqrt(rr2);
+      } else if (!(rr2 > P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
+        // est_lb = ||r_m|| / (||x_m|| theta^{1/2}), theta >= theta_min(T_m), is a lower bound of est
+        need = 1;
+        pfac = sqrt(rr2) * rsqrt(energy);  // ||r_m|| / ||x_m||
+        err = pfac * rsqrt(theta);
+      }
+    }
+    if (lane == 0) {
+      if (status != GMRF_ERR_NOT_SPD && status != GMRF_ERR_NUMERIC) {
         v->d_prev = dinv;
         v->u_prev = u;
       }
@@ -566,8 +600,6 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
       v->err_est = err;
       v->amax = amax;
       v->bmax = bmax;
-      v->beta_last = b;
-      v->vscale = b > 0.0 ? binv : 0.0;
       v->status = status;
       s_pfac = pfac;
       s_need_theta = need;
