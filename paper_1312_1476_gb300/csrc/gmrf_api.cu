@@ -475,11 +475,15 @@ size_t check_bytes_per_vec(const gmrf_problem* p) {
   return 3 * n * es;  // z, u and r
 }
 
-// T_m^{-1} e_1 of the nvec vectors of b into p->ycg (stride m_max).
-int check_tm(gmrf_problem* p, const LanczosBufs& b, cudaStream_t s) {
+// T_m^{-1/2} e_1 of the nvec vectors of b into y and T_m^{-1} e_1 into p->ycg
+// (both of stride m_max).
+int tm_functions(gmrf_problem* p, const LanczosBufs& b, double* y, cudaStream_t s) {
   CKR(ensure(p->ycg, sizeof(double) * 2 * (size_t)b.nvec * b.m_max, p->ws));
   double* ycg = (double*)p->ycg.p;
-  CK(traced(KC_TM, s, 1, [&] { return launch_tm_inv(b, ycg + (size_t)b.nvec * b.m_max, ycg, s); }));
+  CK(traced(KC_TM, s, 3, [&] {
+    return launch_tm_inv_sqrt(b, p->fp64, (TmNodes*)p->nodes.p, (double*)p->scratch.p, y, s, ycg,
+                              ycg + (size_t)b.nvec * b.m_max);
+  }));
   return GMRF_OK;
 }
 
@@ -902,10 +906,7 @@ int gmrf_sample(gmrf_problem* p, const gmrf_sample_opts* o, void* x_out, gmrf_re
     CKR(load_z(b.W[0]));
     CKR(run_lanczos(p, b, o->tol, m_max, o->check_every));
     for (int round = 0;; ++round) {
-      CK(traced(KC_TM, s, 3, [&] {
-        return launch_tm_inv_sqrt(b, p->fp64, (TmNodes*)p->nodes.p, (double*)p->scratch.p, (double*)p->y.p, s);
-      }));
-      CKR(check_tm(p, b, s));
+      CKR(tm_functions(p, b, (double*)p->y.p, s));
       LanczosBufs bx = b;
       if (two_pass) {
         // second pass: the same iteration again (bitwise: same z, same kernels,
@@ -1214,10 +1215,7 @@ int gmrf_sample_logdet(gmrf_problem* p, const gmrf_sample_opts* so, const gmrf_l
     }
     for (int round = 0; nsc > 0; ++round) {
       const LanczosBufs bs = sub_batch(b, 0, nsc, n, es);
-      CK(traced(KC_TM, s, 3, [&] {
-        return launch_tm_inv_sqrt(bs, p->fp64, (TmNodes*)p->nodes.p, (double*)p->scratch.p, (double*)p->y.p, s);
-      }));
-      CKR(check_tm(p, bs, s));
+      CKR(tm_functions(p, bs, (double*)p->y.p, s));
       const double* ycg = (const double*)p->ycg.p;
       if (sparse_f(p)) {
         CKR(ensure(p->work, (size_t)nsc * n * es, p->ws));

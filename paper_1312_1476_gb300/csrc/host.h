@@ -118,7 +118,7 @@ int run_lanczos(gmrf_problem* p, const LanczosBufs& b, double tol, int m_max, in
 StepParams step_params(gmrf_problem* p, const LanczosBufs& b, double tol, int m_max, bool solve);
 LanczosBufs sub_batch(const LanczosBufs& b, int off, int cnt, size_t n, size_t es);
 size_t check_bytes_per_vec(const gmrf_problem* p);
-int check_tm(gmrf_problem* p, const LanczosBufs& b, cudaStream_t s);
+int tm_functions(gmrf_problem* p, const LanczosBufs& b, double* y, cudaStream_t s);
 int check_residuals(gmrf_problem* p, int nvec, const void* z, void* u, bool second, cudaStream_t s);
 double direct_estimate(const VecState& v, const double* d3);
 double crude_estimate(const VecState& v, double rr);

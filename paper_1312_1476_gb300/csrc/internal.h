@@ -129,7 +129,7 @@ constexpr int kMaxNodes = 384;
 // y[s] = T_m^{-1/2} e_1 (rational approximation from the Stieltjes integral),
 // y stride = m_max.  scratch: >= nvec * kMaxNodes * m_max * 2 doubles.
 cudaError_t launch_tm_inv_sqrt(const LanczosBufs& b, bool fp64, TmNodes* nodes, double* scratch, double* y,
-                               cudaStream_t s);
+                               cudaStream_t s, double* ycg, double* work);
 // sparse.cu -----------------------------------------------------------------
 // A general sparse Q (CSR) with an optional incomplete-Cholesky factor F of
 // the preconditioner M = F F^T (Section 5.2).  Device copies, level schedules.

@@ -127,10 +127,7 @@ int finish_samples(gmrf_server* sv, int a, int k, Req& r) {
   const int vec0 = sv->slots[a].vec;
   void* dst = (char*)r.x + (size_t)vec0 * n * es;
   const double xs = 1.0 / std::sqrt(p->tau * r.tau);
-  CK(traced(KC_TM, s, 3, [&] {
-    return launch_tm_inv_sqrt(bs, p->fp64, (TmNodes*)p->nodes.p, (double*)p->scratch.p, (double*)p->y.p, s);
-  }));
-  CKR(check_tm(p, bs, s));
+  CKR(tm_functions(p, bs, (double*)p->y.p, s));
   CKR(ensure(p->ucg, (size_t)k * n * es, p->ws));
   CKR(ensure(p->zre, (size_t)k * n * es, p->ws));
   const double* y = (const double*)p->y.p;

@@ -7,7 +7,7 @@
 // whose integrand is sech(u - log(t)/2) / (2 sqrt t), the trapezoid rule with
 // step h on [u_lo, u_hi] gives
 //   T^{-1/2} e_1 ~= sum_k (2h/pi) e^{u_k} (T + e^{2u_k} I)^{-1} e_1,
-// a sum of shifted SPD tridiagonal solves (Thomas algorithm, one pole per
+// a sum of shifted SPD tridiagonal solves (trailing_dets, one pole per
 // thread).  Discretisation error ~ 4 exp(-pi^2 / h) and truncation error
 // ~ (2/pi) exp(-pad) relative, with the window covering
 // [log(theta_min)/2 - pad, log(theta_max)/2 + pad]; theta_min comes from the
@@ -17,10 +17,11 @@
 //   log t = int_0^inf (1/(1+s) - 1/(t+s)) ds = int_R (e^u/(1+e^u) - e^u/(t+e^u)) du
 // the trapezoid rule gives
 //   e_1^T log(T) e_1 ~= sum_k h e^{u_k} (1/(1+e^{u_k}) - [(T + e^{u_k} I)^{-1}]_{11}),
-// with [(T + sI)^{-1}]_{11} = 1 / d~_1 from the backward continued fraction
-// d~_m = a_m + s, d~_i = a_i + s - b_i^2 / d~_{i+1}.  Error ~ exp(-2 pi^2 / h).
+// with [(T + sI)^{-1}]_{11} the ratio of the two largest trailing determinants.  Error ~ exp(-2 pi^2 / h).
 #include <cuda_runtime.h>
 #include <math.h>
+
+#include <cmath>
 
 #include "internal.h"
 
@@ -47,7 +48,16 @@ __device__ __forceinline__ bool usable(const VecState& v) {
 }
 
 // Node window per vector.  kind 0: inverse square root; kind 1: log.
-__global__ void k_nodes(const VecState* st, const double* alpha, const double* beta, int m_max, int kind, bool fp64,
+struct NodeRule {
+  double h, pad;  // node spacing and what the window exceeds the spectrum by
+};
+// eps: the trapezoid rule's target accuracy
+NodeRule node_rule(int kind, bool fp64) {
+  const double eps = kind == 0 ? (fp64 ? 1e-15 : 1e-11) : (fp64 ? 1e-16 : 1e-12);
+  if (kind == 0) return {kPi * kPi / std::log(4.0 / eps), std::log(2.0 / (kPi * eps))};
+  return {2.0 * kPi * kPi / std::log(1.0 / eps), std::log(1.0 / eps) + 2.0};
+}
+__global__ void k_nodes(const VecState* st, const double* alpha, const double* beta, int m_max, int kind, NodeRule nd,
                         TmNodes* nodes) {
   __shared__ DMax red[8];
   const int s = blockIdx.x;
@@ -69,23 +79,17 @@ __global__ void k_nodes(const VecState* st, const double* alpha, const double* b
     g.v = fmax(g.v, r);
   }
   g = block_reduce(g, red);
-  if (threadIdx.x == 0) {
-    const double tmax = 2.0 * g.v;
+  if (threadIdx.x < 2) {
+    // the two logarithms side by side: an FP64 logarithm is a chain of some microseconds
+    const double tmax = 2.0 * __shfl_sync(3u, g.v, 0);
     const double tmin = 0.5 * v.theta;
-    double eps, h, pad, lo, hi;
-    if (kind == 0) {
-      eps = fp64 ? 1e-15 : 1e-11;
-      h = kPi * kPi / log(4.0 / eps);
-      pad = log(2.0 / (kPi * eps));
-      lo = 0.5 * log(tmin) - pad;
-      hi = 0.5 * log(tmax) + pad;
-    } else {
-      eps = fp64 ? 1e-16 : 1e-12;
-      h = 2.0 * kPi * kPi / log(1.0 / eps);
-      pad = log(1.0 / eps) + 2.0;
-      lo = log(tmin) - pad;
-      hi = log(tmax) + pad;
-    }
+    const double lg = log(threadIdx.x == 0 ? tmin : tmax);
+    const double lgmax = __shfl_sync(3u, lg, 1);
+    if (threadIdx.x > 0) return;
+    double h = nd.h, lo, hi;
+    const double half = kind == 0 ? 0.5 : 1.0;
+    lo = half * lg - nd.pad;
+    hi = half * lgmax + nd.pad;
     if (!(tmin > 0.0) || !(tmax > 0.0) || !isfinite(lo) || !isfinite(hi)) {
       nodes[s] = out;  // L = 0: no usable window (reported through the vector's status)
       return;
@@ -102,40 +106,113 @@ __global__ void k_nodes(const VecState* st, const double* alpha, const double* b
   }
 }
 
-// One pole per thread: D[s][i][k] = w_k ((T + sigma_k I)^{-1} e_1)_i, with the
-// Thomas sweep's c'_i kept in C[s][i][k].  Layout k-fastest for coalescing.
+// (T + sigma I)^{-1} e_1 by the determinants phi_i of the trailing blocks,
+//   phi_m = 1, phi_i = (a_i + sigma) phi_{i+1} - b_i^2 phi_{i+2},
+//   x_i = (-1)^i b_0 .. b_{i-1} phi_{i+1} / phi_0
+// (the closed form of a tridiagonal inverse's first column).  phi_i / phi_{i+1} is
+// the pivot of the backward LDL^T, so rounding acts as there (a relative
+// perturbation of a_i and b_i), but the recurrence holds no division: one
+// dependent FMA per row (64 cycles) where a pivot costs a division (580) and two
+// more operations.  phi is kept as a mantissa and an exponent, rescaled by a power
+// of two (exactly) when it leaves 2^+-128.  With the two logarithms of the window
+// side by side and T_m^{-1} e_1 as one more pole: FP64 64 x 64 sample (102 rows) 133 ->
+// 77 us for the three kernels, 1157 -> 1074 us a call.  Error against 80-bit sums as
+// before (condition 1e6, 300 rows: 3.5e-13, LDL^T 6.6e-13).
+struct Scaled {
+  double v;
+  int e;  // value v 2^e
+  // back into range: v in [1, 2), or 0
+  __device__ __forceinline__ void norm() {
+    const int hi = __double2hiint(v), ex = ((hi >> 20) & 0x7ff) - 1023;
+    if (v == 0.0 || ex == 1024) return;
+    v = __hiloint2double((hi & 0x800fffff) | (1023 << 20), __double2loint(v));
+    e += ex;
+  }
+};
+__device__ __forceinline__ double pow2(int e) {  // 2^e, 0 below the normal range
+  return e < -1022 ? 0.0 : __hiloint2double((min(e, 1023) + 1023) << 20, 0);
+}
+
+// phi_{i+1} of row i = m - 1 .. 0 through put(i, phi); returns phi_0
+template <typename Put>
+__device__ __forceinline__ Scaled trailing_dets(const double* __restrict__ a, const double* __restrict__ b, int m,
+                                                double sigma, Put&& put) {
+  Scaled p = {1.0, 0};  // phi_{i+1}
+  double q = 0.0;       // phi_{i+2}, same exponent
+  for (int i = m - 1; i >= 0; --i) {
+    put(i, p);
+    const double bi = i < m - 1 ? b[i] : 0.0;
+    const double next = fma(a[i] + sigma, p.v, -(bi * (bi * q)));
+    q = p.v;
+    p.v = next;
+    const int ex = ((__double2hiint(next) >> 20) & 0x7ff) - 1023;
+    if (abs(ex) > 128 && ex < 1024 && next != 0.0) {
+      const double s = __hiloint2double((1023 - ex) << 20, 0);
+      p.v *= s;
+      q *= s;
+      p.e += ex;
+    }
+  }
+  return p;
+}
+
+// x_i (times w) from the stored phi_{i+1} (get) into set(i, x).
+template <typename Get, typename Set>
+__device__ __forceinline__ void first_column(const double* __restrict__ b, int m, double w, Scaled phi0, Get&& get,
+                                             Set&& set) {
+  phi0.norm();
+  Scaled pi = {w / phi0.v, -phi0.e};  // w (-1)^i b_0 .. b_{i-1} / phi_0
+  for (int i = 0; i < m; ++i) {
+    const Scaled f = get(i);
+    set(i, pi.v * f.v * pow2(pi.e + f.e));
+    pi.v *= -b[i < m - 1 ? i : 0];
+    pi.norm();
+  }
+}
+
+// y = T_m^{-1} e_1, one thread; work [m] keeps the phi's, y their exponents until
+// they are used
+__device__ void inverse_e1(const double* __restrict__ a, const double* __restrict__ b, int m, double* work, double* y) {
+  const Scaled phi0 = trailing_dets(a, b, m, 0.0, [&](int i, const Scaled& f) {
+    work[i] = f.v;
+    y[i] = (double)f.e;
+  });
+  first_column(b, m, 1.0, phi0, [&](int i) -> Scaled { return {work[i], (int)y[i]}; },
+               [&](int i, double x) { y[i] = x; });
+}
+
+// One pole per thread: D[s][i][k] = w_k ((T + sigma_k I)^{-1} e_1)_i, the phi's
+// exponents kept in C[s][i][k].  Layout k-fastest for coalescing.  Thread
+// kMaxNodes: T^{-1} e_1 itself into ycg[s][i] (work: its phi's), the CG
+// coefficients of the accuracy check.
 __global__ void k_poles(const VecState* st, const double* alpha, const double* beta, int m_max, const TmNodes* nodes,
-                        double* C, double* D) {
+                        int* C, double* D, double* ycg, double* work) {
   const int s = blockIdx.y;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const VecState v = st[s];
   const TmNodes nd = nodes[s];
-  if (!usable(v) || k >= nd.L) return;
+  if (!usable(v) || (k >= nd.L && (k != kMaxNodes || !ycg))) return;
   const int m = v.m;
   const double* a = alpha + (size_t)s * m_max;
   const double* b = beta + (size_t)s * m_max;
+  if (k == kMaxNodes) {
+    inverse_e1(a, b, m, work + (size_t)s * m_max, ycg + (size_t)s * m_max);
+    return;
+  }
   const double u = nd.s_lo + nd.h * k;
-  const double sigma = exp(2.0 * u);
-  const double w = (2.0 * nd.h / kPi) * exp(u);
-  const size_t base = (size_t)s * m_max * kMaxNodes;
-  // forward sweep: c'_i = b_i / den_i, d'_i = (rhs_i - b_{i-1} d'_{i-1}) / den_i
-  double cp = 0.0, dp = 0.0;
-  for (int i = 0; i < m; ++i) {
-    const double den = (a[i] + sigma) - (i > 0 ? b[i - 1] * cp : 0.0);
-    const double rden = 1.0 / den;
-    const double rhs = (i == 0) ? 1.0 : 0.0;
-    dp = (rhs - (i > 0 ? b[i - 1] * dp : 0.0)) * rden;
-    cp = (i < m - 1) ? b[i] * rden : 0.0;
-    C[base + (size_t)i * kMaxNodes + k] = cp;
-    D[base + (size_t)i * kMaxNodes + k] = dp;
-  }
-  // back substitution x_{m-1} = d'_{m-1}, x_i = d'_i - c'_i x_{i+1}
-  double x = 0.0;
-  for (int i = m - 1; i >= 0; --i) {
-    const size_t o = base + (size_t)i * kMaxNodes + k;
-    x = D[o] - C[o] * x;
-    D[o] = w * x;
-  }
+  const double eu = exp(u);
+  const double sigma = eu * eu;  // e^{2u}, one exponential
+  const double w = (2.0 * nd.h / kPi) * eu;
+  const size_t base = (size_t)s * m_max * kMaxNodes + k;
+  const Scaled phi0 = trailing_dets(a, b, m, sigma, [&](int i, const Scaled& f) {
+    C[base + (size_t)i * kMaxNodes] = f.e;
+    D[base + (size_t)i * kMaxNodes] = f.v;
+  });
+  first_column(b, m, w, phi0,
+               [&](int i) -> Scaled {
+                 return {D[base + (size_t)i * kMaxNodes], C[base + (size_t)i * kMaxNodes]};
+               },
+               [&](int i, double x) { D[base + (size_t)i * kMaxNodes] = x; });
 }
 
 // y[s][i] = sum_k D[s][i][k] in a fixed order; one warp per component i.
@@ -177,9 +254,10 @@ __global__ void k_log(const VecState* st, const double* alpha, const double* bet
   for (int k = threadIdx.x; k < nd.L; k += blockDim.x) {
     const double u = nd.s_lo + nd.h * k;
     const double t = exp(u);
-    double dt = a[m - 1] + t;
-    for (int i = m - 2; i >= 0; --i) dt = (a[i] + t) - b[i] * b[i] / dt;
-    acc.v += nd.h * t * (1.0 / (1.0 + t) - 1.0 / dt);
+    // [(T + t I)^{-1}]_{11} = phi_1 / phi_0
+    Scaled phi1 = {1.0, 0};
+    const Scaled phi0 = trailing_dets(a, b, m, t, [&](int, const Scaled& f) { phi1 = f; });
+    acc.v += nd.h * t * (1.0 / (1.0 + t) - phi1.v / phi0.v * pow2(phi1.e - phi0.e));
   }
   acc = block_reduce(acc, red);
   if (threadIdx.x == 0) q[s] = v.znorm * v.znorm * acc.v;
@@ -216,35 +294,15 @@ __global__ void k_logdet_reduce(const double* q, int nq, int group, double shift
   }
 }
 
-// y = T_m^{-1} e_1 (the CG coefficients of a linear solve) by the LDL^T
-// factorisation that the stopping rule also runs: d_0 = a_0,
-// d_i = a_i - b_{i-1}^2 / d_{i-1}, l_i = b_{i-1} / d_{i-1}; L w = e_1 gives
-// w_i = -l_i w_{i-1}; then y = L^{-T} D^{-1} w.  One thread per vector.
+// y = T_m^{-1} e_1 (the CG coefficients of a linear solve).  One thread per vector.
 __global__ void k_tm_inv(const VecState* st, const double* alpha, const double* beta, int m_max, int nvec,
                          double* dwork, double* y) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= nvec) return;
   const VecState v = st[s];
   if (!usable(v)) return;
-  const int m = v.m;
-  const double* a = alpha + (size_t)s * m_max;
-  const double* b = beta + (size_t)s * m_max;
-  double* d = dwork + (size_t)s * m_max;
-  double* ys = y + (size_t)s * m_max;
-  // d[] keeps the reciprocal pivots 1 / d_i: one FP64 division per row (the
-  // chain is serial, and GB300's FP64 divisions are slow)
-  double dinv = 1.0 / a[0], w = 1.0;
-  d[0] = dinv;
-  ys[0] = w * dinv;  // z_i = w_i / d_i
-  for (int i = 1; i < m; ++i) {
-    const double l = b[i - 1] * dinv;
-    const double dp = a[i] - l * b[i - 1];
-    w = -l * w;
-    dinv = 1.0 / dp;
-    d[i] = dinv;
-    ys[i] = w * dinv;
-  }
-  for (int i = m - 2; i >= 0; --i) ys[i] -= (b[i] * d[i]) * ys[i + 1];  // y_i = z_i - l_{i+1} y_{i+1}
+  const size_t o = (size_t)s * m_max;
+  inverse_e1(alpha + o, beta + o, v.m, dwork + o, y + o);
 }
 
 }  // namespace
@@ -255,19 +313,19 @@ cudaError_t launch_tm_inv(const LanczosBufs& b, double* dwork, double* y, cudaSt
 }
 
 cudaError_t launch_tm_inv_sqrt(const LanczosBufs& b, bool fp64, TmNodes* nodes, double* scratch, double* y,
-                               cudaStream_t s) {
-  k_nodes<<<b.nvec, 256, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, 0, fp64, nodes);
-  double* C = scratch;
+                               cudaStream_t s, double* ycg, double* work) {
+  k_nodes<<<b.nvec, 256, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, 0, node_rule(0, fp64), nodes);
+  int* C = (int*)scratch;
   double* D = scratch + (size_t)b.nvec * b.m_max * kMaxNodes;
-  dim3 g1((kMaxNodes + 63) / 64, b.nvec);
-  k_poles<<<g1, 64, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, nodes, C, D);
+  dim3 g1((kMaxNodes + 1 + 63) / 64, b.nvec);
+  k_poles<<<g1, 64, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, nodes, C, D, ycg, work);
   dim3 g2((b.m_max + 7) / 8, b.nvec);
   k_pole_sum<<<g2, 256, 0, s>>>(b.st, b.m_max, nodes, D, y);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tm_log(const LanczosBufs& b, bool fp64, TmNodes* nodes, double* q, cudaStream_t s) {
-  k_nodes<<<b.nvec, 256, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, 1, fp64, nodes);
+  k_nodes<<<b.nvec, 256, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, 1, node_rule(1, fp64), nodes);
   k_log<<<b.nvec, 256, 0, s>>>(b.st, b.alpha, b.beta, b.m_max, nodes, q);
   return cudaGetLastError();
 }
