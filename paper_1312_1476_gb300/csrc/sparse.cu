@@ -235,9 +235,8 @@ struct SpArgs {
 // of n, side by side; x (the second of them) receives the result.  Round by
 // round, every row of the round is a dot product over positions of sm, a group
 // of lanes per row summed by shuffles, with a barrier after the last round of a
-// merged level.  The records run two rounds ahead and the entries of the next
-// round are loaded before this one's sums and barrier, so the chain of a level
-// holds no global load.
+// merged level.  Entries are loaded two rounds ahead (a round takes less than an L2
+// round trip) and records four, so the chain of a level holds no global load.
 constexpr int kTriRegs = 8;  // entries of a lane loaded ahead; longer rows read the rest in place
 
 template <typename T>
@@ -255,46 +254,57 @@ __device__ __forceinline__ void tri_solve(const SpArgs<T>& a, int dir, const T* 
     const int4* p = reinterpret_cast<const int4*>(rec) + 2 * min(r, nr - 1);
     return {__ldg(p), __ldg(p + 1)};
   };
-  int c[kTriRegs];
-  T v[kTriRegs];
-  int row = -1;
-  auto load_entries = [&](const Rec& q) {
+  struct Slots {
+    int c[kTriRegs];
+    T v[kTriRegs];
+    int row;
+  };
+  auto load_entries = [&](const Rec& q, Slots& S) {
     if (tid >= q.a.z) return;
     const int grp = tid >> q.a.w;
-    row = grp < q.b.y ? __ldg(rows + q.b.x + grp) : -1;
+    S.row = grp < q.b.y ? __ldg(rows + q.b.x + grp) : -1;
 #pragma unroll
     for (int k = 0; k < kTriRegs; ++k) {
       if (k < q.a.y) {
-        c[k] = __ldg(col + q.a.x + k * q.a.z + tid);
-        v[k] = __ldg(val + q.a.x + k * q.a.z + tid);
+        S.c[k] = __ldg(col + q.a.x + k * q.a.z + tid);
+        S.v[k] = __ldg(val + q.a.x + k * q.a.z + tid);
       }
     }
   };
-  Rec cur = load_rec(0), nxt = load_rec(1);
-  load_entries(cur);
-  for (int r = 0; r < nr; ++r) {
-    const Rec q = cur;
+  // round r: its entries in S, then those of round r + 2 into S
+  auto round = [&](int r, const Rec& q, const Rec& q2, Slots& S) {
     const bool on = tid < q.a.z;  // whole warps
     T s0 = 0, s1 = 0;
     if (on) {
 #pragma unroll
       for (int k = 0; k < kTriRegs; ++k)
-        if (k < q.a.y && c[k] >= 0) (k & 1 ? s1 : s0) += v[k] * sm[c[k]];
+        if (k < q.a.y && S.c[k] >= 0) (k & 1 ? s1 : s0) += S.v[k] * sm[S.c[k]];
       for (int k = kTriRegs; k < q.a.y; ++k) {
         const int ck = __ldg(col + q.a.x + k * q.a.z + tid);
         if (ck >= 0) s0 += __ldg(val + q.a.x + k * q.a.z + tid) * sm[ck];
       }
     }
-    const int i = row;
-    cur = nxt;
-    nxt = load_rec(r + 2);
-    if (r + 1 < nr) load_entries(cur);
+    const int i = S.row;
+    if (r + 2 < nr) load_entries(q2, S);
     if (on) {
       T acc = s0 + s1;
       for (int off = (1 << q.a.w) >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
       if (i >= 0 && (tid & ((1 << q.a.w) - 1)) == 0) x[i] = acc;
     }
     if (q.b.z) __syncthreads();
+  };
+  Slots A, B;
+  A.row = B.row = -1;
+  Rec q0 = load_rec(0), q1 = load_rec(1), q2 = load_rec(2), q3 = load_rec(3);
+  load_entries(q0, A);
+  if (nr > 1) load_entries(q1, B);
+  for (int r = 0; r < nr; r += 2) {
+    round(r, q0, q2, A);
+    if (r + 1 < nr) round(r + 1, q1, q3, B);
+    q0 = q2;
+    q1 = q3;
+    q2 = load_rec(r + 4);
+    q3 = load_rec(r + 5);
   }
 }
 
@@ -567,7 +577,7 @@ void tri_schedule(int n, const std::vector<int>& rows, const std::vector<int>& l
                   const std::vector<int>& col, const std::vector<double>& val, const std::vector<double>& dg, int b0,
                   int x0, TriHost& out) {
   const int nlev = (int)lptr.size() - 1;
-  typedef std::vector<std::pair<int, double>> Expr;  // (position, coefficient), ascending
+  typedef std::vector<std::pair<int, double>> Expr;  // (position, coefficient)
   std::vector<Expr> expr((size_t)n);  // of the rows of the merged level being built
   std::vector<int> in_block((size_t)n, -1);
   std::vector<double> acc((size_t)std::max(b0, x0) + n, 0.0);
@@ -592,7 +602,6 @@ void tri_schedule(int n, const std::vector<int>& rows, const std::vector<int>& l
       else
         add(x0 + k, -val[(size_t)q]);
     }
-    std::sort(used.begin(), used.end());
     e.clear();
     for (int at : used) e.emplace_back(at, acc[(size_t)at] / dg[(size_t)i]);
   };
