@@ -254,20 +254,33 @@ __device__ __forceinline__ typename Dots<T>::S warp_sum3(const Dots<T>& v) {
   return k;
 }
 
-// Sum over the first nw warps of the block, in a fixed order; the result is
-// valid in every lane of warp 0.  Every thread of the block calls it, and a
-// barrier has to come before `scratch` is used again.
-template <typename T>
-__device__ __forceinline__ Dots<T> reduce_warps(const Dots<T>& v, Dots<T>* scratch, int nw) {
+// The threads that run a sum or the end of a step together: the whole block, or
+// the first N threads of a larger one.
+struct BlockThreads {
+  static __device__ __forceinline__ void sync() { __syncthreads(); }
+  static __device__ __forceinline__ int count() { return (int)(blockDim.x * blockDim.y * blockDim.z); }
+};
+template <int N>
+struct FirstThreads {
+  static __device__ __forceinline__ void sync() { asm volatile("bar.sync 1, %0;" ::"n"(N) : "memory"); }
+  static __device__ __forceinline__ int count() { return N; }
+};
+
+// Sum over the first nw warps of a group of warps, in a fixed order; the result is
+// valid in every lane of the group's warp 0.  `warp` is the caller's place in its
+// group.  Every thread of `Threads` calls it, and a barrier has to come before
+// `scratch` is used again.
+template <typename T, typename Threads = BlockThreads>
+__device__ __forceinline__ Dots<T> reduce_group(const Dots<T>& v, Dots<T>* scratch, int nw, int warp) {
   typedef typename Dots<T>::S S;
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int lane = tid & 31, warp = tid >> 5;
+  const int lane = tid & 31;
   S k = warp < nw ? warp_sum3(v) : S();
   if (nw > 1) {
     S* sc = reinterpret_cast<S*>(scratch);  // [warp][3]
     const int f = lane == 0 ? 0 : (lane == 8 ? 1 : 2);
     if (warp < nw && (lane == 0 || lane == 8 || lane == 16)) sc[warp * 3 + f] = k;
-    __syncthreads();
+    Threads::sync();
     if (warp == 0) {
       // lane 8 f + i adds the warps i, i + 8, ...
       const int g = min(lane >> 3, 2), i = lane & 7;
@@ -282,6 +295,11 @@ __device__ __forceinline__ Dots<T> reduce_warps(const Dots<T>& v, Dots<T>* scrat
   r.s2 = sum_from(k, 8);
   r.s3 = sum_from(k, 16);
   return r;
+}
+template <typename T, typename Threads = BlockThreads>
+__device__ __forceinline__ Dots<T> reduce_warps(const Dots<T>& v, Dots<T>* scratch, int nw) {
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  return reduce_group<T, Threads>(v, scratch, nw, tid >> 5);
 }
 template <typename T>
 __device__ __forceinline__ Dots<T> block_sum(const Dots<T>& v, Dots<T>* scratch) {
@@ -364,10 +382,11 @@ __device__ __forceinline__ int sturm_count(const float* __restrict__ af, const f
 // geometric grid below `hi` (an upper bound).  All threads of the block call
 // it; the result is returned to every thread.  Relative resolution 3e-4 or
 // better, whatever the block's size, ample for the bound's lambda_min^{-1/2}.
+template <typename Threads>
 __device__ __noinline__ static double smallest_ritz(const float* af, const float* b2f, int m, double hi_in, int* s_int,
                                 float* s_flt) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int nt = blockDim.x * blockDim.y * blockDim.z;
+  const int nt = Threads::count();
   float hi = (float)(hi_in * 1.0001) + 1e-30f;
   float lo = hi * 1e-8f;
   for (int round = 0; round < 8; ++round) {
@@ -377,10 +396,10 @@ __device__ __noinline__ static double smallest_ritz(const float* af, const float
     if (tid == nt - 1) p = hi;
     int c = sturm_count(af, b2f, m, p);
     if (tid == 0) s_int[0] = nt;  // first index with count >= 1
-    __syncthreads();
+    Threads::sync();
     if (c >= 1) atomicMin(&s_int[0], tid);
     int c_lo = (tid == 0) ? sturm_count(af, b2f, m, lo) : 0;
-    __syncthreads();
+    Threads::sync();
     if (tid == 0) {
       int t = s_int[0];
       float nlo = lo, nhi = hi;
@@ -403,11 +422,11 @@ __device__ __noinline__ static double smallest_ritz(const float* af, const float
       s_flt[1] = nhi;
       s_int[1] = again;
     }
-    __syncthreads();
+    Threads::sync();
     lo = s_flt[0];
     hi = s_flt[1];
     int again = s_int[1];
-    __syncthreads();
+    Threads::sync();
     if (again == 0 || again == 3) break;
   }
   return (double)hi;
@@ -494,13 +513,17 @@ __device__ __forceinline__ double step_b2(double a, double s2, double s3, double
 // With warp_sum3 and publish(), before and now: FP64 64 x 64 step 17.2 -> 11.7 us
 // (one vector; 12.7 with all of it in one warp), 93 -> 48 us (256 vectors); 512 x 512
 // row-last pass, 320 vectors, 346 -> 317 us.
-template <typename T>
-__device__ static void finish_step(const StepParams& P, int j, int s, const Dots<T>* __restrict__ partials, int nblk,
+// The records come from rec(b), and rec's Threads run it; where the caller keeps the
+// iteration in one kernel (Rec::kept), the state is in shared memory, alpha, beta, 1 / beta and the
+// status also go to rec's shared copy, and the caller stores alpha_j and beta_j.
+template <typename T, typename Rec>
+__device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int s, const Rec& rec, int nblk,
                             VecState* __restrict__ st, double* __restrict__ alpha, double* __restrict__ beta,
                             float* __restrict__ alpha_f, float* __restrict__ beta2_f, Dots<T>* red_scratch,
-                            int* s_int, float* s_flt, double b2_direct = -1.0) {
+                            int* s_int, float* s_flt, double b2_direct) {
+  typedef typename Rec::Threads Threads;
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-  const int nt = blockDim.x * blockDim.y * blockDim.z;
+  const int nt = Threads::count();
   const int warp = tid >> 5, lane = tid & 31;
   const int nw = min(nt >> 5, (nblk + 31) >> 5);
   __shared__ int s_need_theta;
@@ -515,10 +538,10 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
   Dots<T> acc;
   acc.zero();
   if (warp < nw)
-    for (int b = tid; b < nblk; b += 32 * nw) acc.merge(load_partial(partials + (size_t)s * nblk + b));
-  acc = reduce_warps(acc, red_scratch, nw);
+    for (int b = tid; b < nblk; b += 32 * nw) acc.merge(rec(b));
+  acc = reduce_warps<T, Threads>(acc, red_scratch, nw);
   if (tid == 0) acc.get(s_sum[0], s_sum[1], s_sum[2]);
-  __syncthreads();
+  Threads::sync();
   const double a = s_sum[0];
   // warp 0: alpha_j, beta_j and 1 / beta_j, which the next step waits for
   if (warp == 0) {
@@ -529,10 +552,14 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
     b = fma(fma(-b, b, b2), 0.5 * y, b);
     if (!(b2 < 1e300) || b2 < 1e-290) b = b2 > 0.0 ? sqrt(b2) : 0.0;  // where b2 or y leave the range (or are no numbers)
     if (lane == 0) {
-      alpha[mo + j] = a;
-      beta[mo + j] = b;
-      alpha_f[mo + j] = (float)a;
-      beta2_f[mo + j] = (float)(b * b);
+      if constexpr (Rec::kept) {
+        rec.keep(a, b, y);
+      } else {
+        alpha[mo + j] = a;
+        beta[mo + j] = b;
+        alpha_f[mo + j] = (float)a;
+        beta2_f[mo + j] = (float)(b * b);
+      }
       v->beta_last = b;
       v->vscale = y;
     }
@@ -601,14 +628,22 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
       v->amax = amax;
       v->bmax = bmax;
       v->status = status;
+      if constexpr (Rec::kept) *rec.status = status;
       s_pfac = pfac;
       s_need_theta = need;
       s_theta_hi = theta;
     }
   }
-  __syncthreads();
+  Threads::sync();
   if (s_need_theta) {
-    double th = smallest_ritz(alpha_f + mo, beta2_f + mo, j + 1, s_theta_hi, s_int, s_flt);
+    if constexpr (Rec::kept) {
+      if (tid == 0) {
+        alpha_f[mo + j] = (float)rec.scalars[0];
+        beta2_f[mo + j] = (float)(rec.scalars[1] * rec.scalars[1]);
+      }
+      Threads::sync();
+    }
+    double th = smallest_ritz<Threads>(alpha_f + mo, beta2_f + mo, j + 1, s_theta_hi, s_int, s_flt);
     if (tid == 0) {
       v->theta = th;
       if (v->status == VS_RUNNING) {
@@ -616,10 +651,29 @@ __device__ static void finish_step(const StepParams& P, int j, int s, const Dots
         v->err_est = est;
         if (est <= P.tol && j + 1 >= v->m_min) v->status = VS_DONE;
         else if (j + 1 >= P.m_max) v->status = GMRF_ERR_NOT_CONVERGED;
+        if constexpr (Rec::kept) *rec.status = v->status;
       }
     }
   }
 }
+
+// the records that the blocks of a vector published
+template <typename T>
+struct PublishedRecords {
+  static constexpr bool kept = false;
+  typedef BlockThreads Threads;
+  const Dots<T>* p;
+  __device__ __forceinline__ Dots<T> operator()(int b) const { return load_partial(p + b); }
+};
+template <typename T>
+__device__ static void finish_step(const StepParams& P, int j, int s, const Dots<T>* __restrict__ partials, int nblk,
+                            VecState* __restrict__ st, double* __restrict__ alpha, double* __restrict__ beta,
+                            float* __restrict__ alpha_f, float* __restrict__ beta2_f, Dots<T>* red_scratch,
+                            int* s_int, float* s_flt, double b2_direct = -1.0) {
+  finish_step_from<T>(P, j, s, PublishedRecords<T>{partials + (size_t)s * nblk}, nblk, st, alpha, beta, alpha_f,
+                      beta2_f, red_scratch, s_int, s_flt, b2_direct);
+}
+
 
 // ------------------------------------------------------------------- Philox
 __device__ __forceinline__ void philox4x32_10(uint32_t c[4], uint32_t k0, uint32_t k1) {

@@ -178,7 +178,19 @@ int worst_status(const VecState* st, int nvec) {
 
 // Runs the Lanczos iteration on the vectors already in W[0].  Returns a
 // gmrf code for launch failures only; per-vector outcomes are in st_host.
+// The grids whose steps one launch runs until its vectors stop; not where something
+// happens after each step (the two-pass accumulation, a timed launch).
+bool resident_steps(const gmrf_problem* p, const LanczosBufs& b) {
+  return !p->sp && p->precond == GMRF_PREC_NONE && !b.Xacc && !trace_timing_enabled() &&
+         stencil2d_resident_eligible(p->g, p->fp64, b.nvec);
+}
+
 int launch_steps(gmrf_problem* p, const LanczosBufs& b, const StepParams& P, int c, cudaStream_t s) {
+  if (resident_steps(p, b)) {
+    CK(traced(KC_STENCIL_STEP, s, 1,
+              [&] { return launch_stencil_step(p->g, p->fp64, p->kappa2.p, p->kappa2_const, b, P, s, c); }));
+    return GMRF_OK;
+  }
   for (int k = 0; k < c; ++k) {
     if (p->sp)
       CK(traced(KC_SPARSE_STEP, s, 1, [&] { return launch_sparse_step(*p->sp, b, P, s); }));
@@ -390,7 +402,8 @@ int run_lanczos(gmrf_problem* p, const LanczosBufs& b, double tol, int m_max, in
     // kernel and the body's launch), and a shorter body wastes fewer steps
     // after the last vector stops (1024^2 headline: 4.24 ms per sample with
     // 8-step bodies, 4.32 with 16, 4.60 with 1, 4.28 host-replayed).
-    CKR(capture_loop(p, b, P, std::min(c, 8)));
+    // Resident steps end by themselves: one launch for all of them.
+    CKR(capture_loop(p, b, P, resident_steps(p, b) ? m_max : std::min(c, 8)));
     if (G.exec) {
       int iters = 0;
       CK(cudaGraphLaunch(G.exec, s));

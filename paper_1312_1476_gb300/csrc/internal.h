@@ -57,8 +57,11 @@ int stencil_blocks_per_vector(const Grid& g);
 // Fused step j of Algorithm 1 with the matrix-free stencil Q: forms v_j,
 // stores it, q_j = Q v_j - beta_{j-1} v_{j-1}, dot products, alpha_j, beta_j,
 // stopping rule.  W[j&1] is read, W[(j+1)&1] written.
+// nsteps > 1, for the grids of stencil2d_resident.cu alone: that many steps, or
+// fewer where a vector stops.
 cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
-                                const LanczosBufs& b, const StepParams& P, cudaStream_t s);
+                                const LanczosBufs& b, const StepParams& P, cudaStream_t s, int nsteps = 1);
+bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec);
 // y = Q v for nvec vectors (no Lanczos bookkeeping).
 cudaError_t launch_stencil_apply(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
                                  const void* v, void* y, int nvec, cudaStream_t s, double scale = 1.0);

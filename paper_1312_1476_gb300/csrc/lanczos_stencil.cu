@@ -29,16 +29,8 @@
 namespace gmrf {
 namespace {
 
-constexpr int TX = 32;
-// Rows of a 2-D tile, two of them a thread's: half the additions of a sum over
-// the block, and half its barriers, per cell.  FP64 tiles are 8 rows, so that a
-// small grid spreads over more SMs (their FP64 lanes bound it), FP32 tiles 16.
-// 64 x 64 periodic, about 26 steps, one vector and 256, 16 rows and one a thread
-// (512 threads) before: FP64 636 -> 588 us and 3119 -> 2732, FP32 514 -> 508 and
-// 1872 -> 1549.
-constexpr int CPT = 2;
-template <typename T>
-__host__ __device__ constexpr int tile_y() { return sizeof(T) == 8 ? 8 : 16; }
+constexpr int TX = kTileX;
+constexpr int CPT = kTileCells;
 
 __device__ __forceinline__ int wrapi(int g, int n) {
   g %= n;
@@ -56,20 +48,19 @@ __device__ __forceinline__ T kap_at(const float* k, T kc, size_t i) {
 template <typename T, int BC, int W>
 __device__ __forceinline__ T bop2(const T* a, int cx, int cy, int gx, int gy, int nx, int ny, T kap) {
   const T c = a[cy * W + cx];
-  T r = kap * c;
-  if (BC != GMRF_BC_NEUMANN || gx > 0) r += c - a[cy * W + cx - 1];
-  if (BC != GMRF_BC_NEUMANN || gx < nx - 1) r += c - a[cy * W + cx + 1];
-  if (BC != GMRF_BC_NEUMANN || gy > 0) r += c - a[(cy - 1) * W + cx];
-  if (BC != GMRF_BC_NEUMANN || gy < ny - 1) r += c - a[(cy + 1) * W + cx];
-  return r;
+  const T l = BC != GMRF_BC_NEUMANN || gx > 0 ? edge(c, a[cy * W + cx - 1]) : (T)0;
+  const T r = BC != GMRF_BC_NEUMANN || gx < nx - 1 ? edge(c, a[cy * W + cx + 1]) : (T)0;
+  const T u = BC != GMRF_BC_NEUMANN || gy > 0 ? edge(c, a[(cy - 1) * W + cx]) : (T)0;
+  const T d = BC != GMRF_BC_NEUMANN || gy < ny - 1 ? edge(c, a[(cy + 1) * W + cx]) : (T)0;
+  return b_cell(kap, c, l, r, u, d);
 }
 
 // STEP = true: fused Lanczos step.  STEP = false: y = Q v (Win = v, Wout = y).
 // SPDE_PLUS_DIAG: Q v = B(B v) + D v with B = kappa_c^2 I + L (constant
 // coefficient, kappa2_const) and D = diag(kappa2 field, or 0).
 template <typename T, int OP, int BC, bool STEP>
-__global__ void __launch_bounds__(TX * tile_y<T>() / CPT) k_stencil2d(StencilArgs<T> a) {
-  constexpr int TY = tile_y<T>(), NT = TX * TY / CPT;
+__global__ void __launch_bounds__(TX * tile2d_y<T>() / CPT) k_stencil2d(StencilArgs<T> a) {
+  constexpr int TY = tile2d_y<T>(), NT = TX * TY / CPT;
   constexpr bool SQ = OP != GMRF_OP_SHIFTED_LAPLACIAN;  // B applied twice
   constexpr int H = SQ ? 2 : 1;
   constexpr int VW = TX + 2 * H, VH = TY + 2 * H;
@@ -123,8 +114,7 @@ __global__ void __launch_bounds__(TX * tile_y<T>() / CPT) k_stencil2d(StencilArg
       const size_t i = (size_t)gx + (size_t)nx * gy;
       const T w = Win[i];
       if (!STEP) val = w;
-      else if (j == 0) val = w * inv_b;
-      else val = (w - coef * Vp[i]) * inv_b;
+      else val = next_v(w, j > 0 ? Vp[i] : (T)0, coef, inv_b, j > 0);
     }
     vs[idx] = val;
   }
@@ -167,7 +157,7 @@ __global__ void __launch_bounds__(TX * tile_y<T>() / CPT) k_stencil2d(StencilArg
     } else {
       const T v = vs[(cy + H) * VW + tx + H];
       T q = qv;
-      if (j > 0) q -= bprev * Vp[i];
+      if (j > 0) q = less(q, bprev, Vp[i]);
       Wout[i] = q;
       Vc[i] = v;
       if (a.P.vb) vb_store1(vb_at(a.P, s, j, a.n, i), (float)v);
@@ -451,8 +441,11 @@ int nz_chunks(const Grid& g, int vx) {
 }
 
 template <typename T, bool STEP>
-cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s) {
-  constexpr int TY = tile_y<T>();
+cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s, int nsteps = 1) {
+  if (STEP && stencil2d_resident_eligible(g, sizeof(T) == 8, nvec))
+    return launch_stencil2d_resident<T>(g, a, nvec, nsteps, s);
+  if (nsteps != 1) return cudaErrorNotSupported;
+  constexpr int TY = tile2d_y<T>();
   dim3 blk(TX, TY / CPT);
   dim3 grd((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, nvec);
   if (g.dim == 3) {
@@ -533,14 +526,14 @@ int stencil_blocks_per_vector(const Grid& g) {
     const int t = stencil3d_tma_eligible(g, false) ? stencil3d_tma_items_per_vector(g) : 0;
     return r > t ? r : t;
   }
-  int r = ((g.nx + TX - 1) / TX) * ((g.ny + tile_y<double>() - 1) / tile_y<double>());
+  int r = ((g.nx + TX - 1) / TX) * ((g.ny + tile2d_y<double>() - 1) / tile2d_y<double>());
   for (int fp64 = 0; fp64 < 2; ++fp64)
     if (stencil2d_strip_eligible(g, fp64 != 0)) r = std::max(r, stencil2d_strip_blocks_per_vector(g, fp64 != 0));
   return r;
 }
 
 cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
-                                const LanczosBufs& b, const StepParams& P, cudaStream_t s) {
+                                const LanczosBufs& b, const StepParams& P, cudaStream_t s, int nsteps) {
   if (fp64) {
     auto a = make_args<double>(g, kappa2, kappa2_const);
     a.W0 = (double*)b.W[0];
@@ -550,7 +543,7 @@ cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, do
     a.st = b.st; a.alpha = b.alpha; a.beta = b.beta; a.alpha_f = b.alpha_f; a.beta2_f = b.beta2_f;
     a.partials = (Dots<double>*)b.partials;
     a.counters = b.counters;
-    return dispatch<double, true>(g, a, b.nvec, s);
+    return dispatch<double, true>(g, a, b.nvec, s, nsteps);
   }
   auto a = make_args<float>(g, kappa2, kappa2_const);
   a.W0 = (float*)b.W[0];
@@ -560,7 +553,7 @@ cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, do
   a.st = b.st; a.alpha = b.alpha; a.beta = b.beta; a.alpha_f = b.alpha_f; a.beta2_f = b.beta2_f;
   a.partials = (Dots<float>*)b.partials;
   a.counters = b.counters;
-  return dispatch<float, true>(g, a, b.nvec, s);
+  return dispatch<float, true>(g, a, b.nvec, s, nsteps);
 }
 
 cudaError_t launch_stencil_apply(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
