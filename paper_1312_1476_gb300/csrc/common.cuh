@@ -363,60 +363,83 @@ __device__ __forceinline__ void vb_store4(__nv_bfloat16* p, float a, float b, fl
   *reinterpret_cast<uint2*>(p) = u;
 }
 
-// Count of eigenvalues of T_m below sigma (Sturm sequence of the LDL^T pivots
-// of T_m - sigma I), in FP32 on float copies of alpha and beta^2.
-__device__ __forceinline__ int sturm_count(const float* __restrict__ af, const float* __restrict__ b2f, int m,
-                                           float sigma) {
-  int cnt = 0;
-  float d = 1.f;
-  for (int i = 0; i < m; ++i) {
-    float a = af[i] - sigma;
-    d = (i == 0) ? a : a - __fdividef(b2f[i - 1], d);
-    if (fabsf(d) < 1e-30f) d = -1e-30f;
-    cnt += (d < 0.f);
+// Whether T_m has an eigenvalue at or below sigma: a leading determinant of
+// T_m - sigma I that is not positive (Sturm sequence), in FP32 on float copies of alpha and
+// beta^2.  The determinants' recurrence takes one dependent FMA per row where the
+// pivots' takes a division; scale (a power of two near 1 / ||T_m||) and a power of two
+// every fourth row keep it in range.
+__device__ __forceinline__ bool ritz_below(const float* __restrict__ af, const float* __restrict__ b2f, int m,
+                                           float sigma, float scale) {
+  float p1 = 1.f, p = (af[0] - sigma) * scale;
+  bool bad = !(p > 0.f);
+  int i = 1;
+  auto row = [&](float a, float b2) {
+    const float n = fmaf((a - sigma) * scale, p, -((b2 * scale) * scale) * p1);
+    p1 = p;
+    p = n;
+    bad |= !(p > 0.f);
+  };
+  for (; i + 4 <= m; i += 4) {
+    float a[4], b2[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      a[k] = af[i + k];
+      b2[k] = b2f[i + k - 1];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) row(a[k], b2[k]);
+    // the power of two that brings the larger of the two near 1 (what follows a
+    // determinant that is not positive does not matter)
+    const int ex = (__float_as_int(fmaxf(p, p1)) >> 23) & 0xff;
+    const float f = __int_as_float(min(max(254 - ex, 1), 254) << 23);
+    p *= f;
+    p1 *= f;
   }
-  return cnt;
+  for (; i < m; ++i) row(af[i], b2f[i - 1]);
+  return bad;
 }
 
 // Smallest eigenvalue of T_m by multisection over the block's threads on a
 // geometric grid below `hi` (an upper bound).  All threads of the block call
 // it; the result is returned to every thread.  Relative resolution 3e-4 or
 // better, whatever the block's size, ample for the bound's lambda_min^{-1/2}.
+// The first window is eight decades below hi, where 256 threads need two rounds, or
+// two, where fewer do unless theta fell by more than that since it was last formed.
 template <typename Threads>
-__device__ __noinline__ static double smallest_ritz(const float* af, const float* b2f, int m, double hi_in, int* s_int,
-                                float* s_flt) {
+__device__ __noinline__ static double smallest_ritz(const float* af, const float* b2f, int m, double hi_in, float scale,
+                                                    int* s_int, float* s_flt) {
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nt = Threads::count();
+  const float window = nt >= 256 ? 1e-8f : 1e-2f;
   float hi = (float)(hi_in * 1.0001) + 1e-30f;
-  float lo = hi * 1e-8f;
-  for (int round = 0; round < 8; ++round) {
-    // points p_t = lo * (hi/lo)^((t+1)/nt), t = 0..nt-1 ; p_{nt-1} = hi
-    float lr = __logf(hi / lo);
-    float p = lo * __expf(lr * (float)(tid + 1) / (float)nt);
+  float lo = hi * window;
+  for (int round = 0; round < 12; ++round) {
+    // points p_t = lo * (hi/lo)^(t/(nt-1)), t = 0..nt-1
+    const float lr = __logf(hi / lo) / (float)(nt - 1);
+    float p = lo * __expf(lr * (float)tid);
+    if (tid == 0) p = lo;
     if (tid == nt - 1) p = hi;
-    int c = sturm_count(af, b2f, m, p);
-    if (tid == 0) s_int[0] = nt;  // first index with count >= 1
+    const bool c = ritz_below(af, b2f, m, p, scale);
+    if (tid == 0) s_int[0] = nt;  // first point with an eigenvalue below
     Threads::sync();
-    if (c >= 1) atomicMin(&s_int[0], tid);
-    int c_lo = (tid == 0) ? sturm_count(af, b2f, m, lo) : 0;
+    if (c) atomicMin(&s_int[0], tid);
     Threads::sync();
     if (tid == 0) {
-      int t = s_int[0];
+      const int t = s_int[0];
       float nlo = lo, nhi = hi;
       int again = 0;
-      if (c_lo >= 1) {          // theta_min below lo: move the window down
+      if (t == 0) {             // theta_min below lo: move the window down
         nhi = lo;
-        nlo = lo * 1e-8f;
+        nlo = lo * window;
         again = (nlo > 1e-35f) ? 2 : 3;
       } else if (t == nt) {     // hi was not an upper bound: widen up
         nlo = hi;
         nhi = hi * 1e4f;
         again = 2;
       } else {
-        nhi = lo * __expf(lr * (float)(t + 1) / (float)nt);
-        if (t == nt - 1) nhi = hi;
-        nlo = (t == 0) ? lo : lo * __expf(lr * (float)t / (float)nt);
-        again = (round == 0 || nhi > nlo * 1.0003f) ? 1 : 0;  // two refinement rounds with 256 threads, three with fewer
+        if (t < nt - 1) nhi = lo * __expf(lr * (float)t);
+        if (t > 1) nlo = lo * __expf(lr * (float)(t - 1));
+        again = (round == 0 || nhi > nlo * 1.0003f) ? 1 : 0;
       }
       s_flt[0] = nlo;
       s_flt[1] = nhi;
@@ -486,8 +509,17 @@ __device__ __forceinline__ Dots<double> load_partial(const Dots<double>* p) {
 
 // beta_j^2 from the three sums, or the caller's
 __device__ __forceinline__ double step_b2(double a, double s2, double s3, double b2_direct) {
-  return b2_direct >= 0.0 ? b2_direct : s2 - 2.0 * a * a + a * a * s3;
+  return b2_direct >= 0.0 ? b2_direct : fma(a * a, s3 - 2.0, s2);
 }
+
+// Tests of doubles on their bits: a comparison takes the FP64 lanes as long as an addition.
+__device__ __forceinline__ long long bits(double x) { return __double_as_longlong(x); }
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool is_positive(double x) { return bits(x) > 0; }  // of a finite x
+// larger of two doubles that are not negative
+__device__ __forceinline__ double larger(double x, double y) { return bits(x) > bits(y) ? x : y; }
+__device__ __forceinline__ double one_sum(df v) { return df_to_double(v); }
+__device__ __forceinline__ double one_sum(double v) { return v; }
 
 // End of a Lanczos step for vector s, run by the last block of that vector
 // (every thread of the block calls it).  Sums the per-block partial dot
@@ -512,7 +544,11 @@ __device__ __forceinline__ double step_b2(double a, double s2, double s3, double
 // Only as many warps as there are partial sums take part in the sum.
 // With warp_sum3 and publish(), before and now: FP64 64 x 64 step 17.2 -> 11.7 us
 // (one vector; 12.7 with all of it in one warp), 93 -> 48 us (256 vectors); 512 x 512
-// row-last pass, 320 vectors, 346 -> 317 us.
+// row-last pass, 320 vectors, 346 -> 317 us.  Comparisons on the bits, beta_j^2 in three
+// operations, a lane per sum where pairs of floats become doubles, and smallest_ritz on
+// determinants (26 us a call at m = 100 with a division per row and two counts in one
+// thread): samples of 64 x 64 in FP64 849 -> 747 us, 61 x 75 x 90 1008 -> 982, 1024 x 1024
+// 3904 -> 3768, 24 slots of 256 x 256 5489 -> 5313.
 // The records come from rec(b), and rec's Threads run it; where the caller keeps the
 // iteration in one kernel (Rec::kept), the state is in shared memory, alpha, beta, 1 / beta and the
 // status also go to rec's shared copy, and the caller stores alpha_j and beta_j.
@@ -528,6 +564,7 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
   const int nw = min(nt >> 5, (nblk + 31) >> 5);
   __shared__ int s_need_theta;
   __shared__ double s_theta_hi, s_pfac;
+  __shared__ float s_scale;
   const size_t mo = (size_t)s * P.m_max;
   VecState* const v = st + s;
   // the state's fields d_prev .. beta_last, one per lane of warp 1 (the only warp
@@ -538,19 +575,24 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
   Dots<T> acc;
   acc.zero();
   if (warp < nw)
-    for (int b = tid; b < nblk; b += 32 * nw) acc.merge(rec(b));
+    if (tid < nblk) {
+      acc = rec(tid);
+      for (int b = tid + 32 * nw; b < nblk; b += 32 * nw) acc.merge(rec(b));
+    }
   acc = reduce_warps<T, Threads>(acc, red_scratch, nw);
-  if (tid == 0) acc.get(s_sum[0], s_sum[1], s_sum[2]);
+  if (tid < 3) s_sum[tid] = one_sum(tid == 0 ? acc.s1 : (tid == 1 ? acc.s2 : acc.s3));  // a lane each
   Threads::sync();
   const double a = s_sum[0];
   // warp 0: alpha_j, beta_j and 1 / beta_j, which the next step waits for
   if (warp == 0) {
     const double b2 = step_b2(a, s_sum[1], s_sum[2], b2_direct);
-    const double y = b2 > 0.0 ? rsqrt(b2) : 0.0;
+    // a number, positive, and neither b2 nor 1 / sqrt(b2) near the ends of the range
+    const bool plain = bits(b2) > bits(1e-290) && bits(b2) < bits(1e300);
+    const double y = plain || b2 > 0.0 ? rsqrt(b2) : 0.0;
     // beta_j = sqrt(b2) from y by one Newton step on the residual b2 - b^2
     double b = b2 * y;
     b = fma(fma(-b, b, b2), 0.5 * y, b);
-    if (!(b2 < 1e300) || b2 < 1e-290) b = b2 > 0.0 ? sqrt(b2) : 0.0;  // where b2 or y leave the range (or are no numbers)
+    if (!plain) b = b2 > 0.0 ? sqrt(b2) : 0.0;
     if (lane == 0) {
       if constexpr (Rec::kept) {
         rec.keep(a, b, y);
@@ -581,12 +623,12 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
       theta = a;
     }
     const double dinv = 1.0 / d;
-    const bool finite = isfinite(a) && isfinite(b2) && isfinite(d);
+    const bool finite = is_finite(a) && is_finite(b2) && is_finite(d);
     int need = 0, status = VS_RUNNING;
     double pfac = 0.0;
-    amax = fmax(amax, fabs(a));
-    if (j > 0) bmax = fmax(bmax, b_prev);
-    if (!finite || d <= 0.0 || a <= 0.0) {
+    amax = larger(amax, fabs(a));
+    if (j > 0) bmax = larger(bmax, b_prev);
+    if (!finite || !is_positive(d) || !is_positive(a)) {
       // the estimate of the last completed step stays on record
       status = finite ? GMRF_ERR_NOT_SPD : GMRF_ERR_NUMERIC;
       if (j > 0) {
@@ -596,20 +638,20 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
     } else {
       const double ud = u * dinv;
       energy += u * ud;
-      const double rr2 = fmax(b2, 0.0) * (ud * ud);  // (||r_m|| / ||z||)^2
+      const double rr2 = (is_positive(b2) ? b2 : 0.0) * (ud * ud);  // (||r_m|| / ||z||)^2
       const double bd = P.bd_tol * (amax + bmax);
-      if (b2 <= bd * bd) {
+      if (bits(b2) <= bits(bd * bd)) {  // bd is not negative; a negative b2 is the smaller one here too
         status = VS_DONE;  // invariant Krylov subspace: x_m is exact
         err = 0.0;
         need = !P.solve;   // theta still wanted for the T_m function of a sample
       } else if (P.solve) {
         // linear solve: x_m = ||z|| V_m T_m^{-1} e_1 is the CG iterate, with
         // relative residual ||r_m|| / ||z|| = beta_m |e_m^T T_m^{-1} e_1|
-        const bool done = rr2 <= P.tol * P.tol;
+        const bool done = bits(rr2) <= bits(P.tol * P.tol);
         if (done) status = VS_DONE;
         else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
         if (status != VS_RUNNING) err = sqrt(rr2);
-      } else if (!(rr2 > P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
+      } else if (bits(rr2) <= bits(P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
         // est_lb = ||r_m|| / (||x_m|| theta^{1/2}), theta >= theta_min(T_m), is a lower bound of est
         need = 1;
         pfac = sqrt(rr2) * rsqrt(energy);  // ||r_m|| / ||x_m||
@@ -632,6 +674,8 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
       s_pfac = pfac;
       s_need_theta = need;
       s_theta_hi = theta;
+      // 1 over the power of two in max |alpha_i|, a scale of T_m
+      s_scale = __int_as_float(min(max(254 - ((__float_as_int((float)amax) >> 23) & 0xff), 1), 253) << 23);
     }
   }
   Threads::sync();
@@ -643,7 +687,7 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
       }
       Threads::sync();
     }
-    double th = smallest_ritz<Threads>(alpha_f + mo, beta2_f + mo, j + 1, s_theta_hi, s_int, s_flt);
+    double th = smallest_ritz<Threads>(alpha_f + mo, beta2_f + mo, j + 1, s_theta_hi, s_scale, s_int, s_flt);
     if (tid == 0) {
       v->theta = th;
       if (v->status == VS_RUNNING) {

@@ -21,8 +21,8 @@
 //
 // Bound: the chain of a step's dependent operations.  FP64 64 x 64 (one vector, 102
 // steps, cycles a step): v_j 670, the cells and their sums 3900 (an FP64 operation of a
-// warp takes its quarter of the SM 64 cycles), the end of the step 5400, the barriers 500 to 700
-// each.  Two cells a thread: with four or eight in fewer warps the call took 973 and
+// warp takes its quarter of the SM 64 cycles), the end of the step 5400 (about 3400
+// since its comparisons left the FP64 lanes), the barriers 500 to 700 each.  Two cells a thread: with four or eight in fewer warps the call took 973 and
 // 1260 us against 808, since an SM's quarters have their own FP64 lanes.  Measured,
 // sample calls with one vector against the one-step kernel: FP64 to 1e-10 64 x 64
 // 1131 -> 859 us, 24 x 24 671 -> 542, 91 x 77 1239 -> 1154; FP32 to 1e-6 731 -> 557,
