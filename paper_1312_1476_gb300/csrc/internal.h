@@ -102,7 +102,7 @@ cudaError_t launch_accumulate_finish(bool fp64, size_t n, const LanczosBufs& b, 
 // r = z - r in place for count elements of float or double.
 cudaError_t launch_resid_form(bool z64, const void* z, bool r64, void* r, size_t count, cudaStream_t s);
 // out[3 s .. 3 s + 2] = (r.r, r.t, t.t) in FP64 sums for nvec vectors [nvec][n]
-// of float or double; part: kResidBlocks * nvec Dots<double> of scratch.
+// of float or double; part: kResidBlocks * nvec Dots<double> of scratch (the most it takes).
 constexpr int kResidBlocks = 128;
 cudaError_t launch_dots3(bool r64, const void* r, const void* t, size_t n, int nvec, void* part, double* out,
                          cudaStream_t s);

@@ -524,10 +524,12 @@ __global__ void k_field_stats(const float* k, size_t n, Dots<float>* part) {
   if (threadIdx.x == 0) part[blockIdx.x] = d;
 }
 __global__ void k_field_final(const Dots<float>* part, int np, double* out4) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  __shared__ Dots<float> red[8];
   Dots<float> d;
   d.zero();
-  for (int b = 0; b < np; ++b) d.merge(part[b]);
+  for (int b = threadIdx.x; b < np; b += blockDim.x) d.merge(part[b]);
+  d = block_reduce(d, red);
+  if (threadIdx.x != 0) return;
   double a, b2, c;
   d.get(a, b2, c);
   out4[0] = b2;
@@ -575,7 +577,7 @@ cudaError_t launch_rng_coloured(bool fp64, int64_t nvec, int64_t n, uint64_t see
 cudaError_t launch_field_stats(const float* k, size_t n, double* out4, cudaStream_t s) {
   Dots<float>* part = reinterpret_cast<Dots<float>*>(out4 + 4);
   k_field_stats<<<kFieldBlocks, 256, 0, s>>>(k, n, part);
-  k_field_final<<<1, 32, 0, s>>>(part, kFieldBlocks, out4);
+  k_field_final<<<1, 256, 0, s>>>(part, kFieldBlocks, out4);
   return cudaGetLastError();
 }
 
@@ -674,10 +676,17 @@ cudaError_t launch_resid_form(bool z64, const void* z, bool r64, void* r, size_t
 
 cudaError_t launch_dots3(bool r64, const void* r, const void* t, size_t n, int nvec, void* part, double* out,
                          cudaStream_t s) {
-  dim3 grd(kResidBlocks, nvec);
+  // A block's end (FP64 additions and conversions in all its warps) costs as much as
+  // several cells of every thread, so small vectors take few blocks.  Sample calls with
+  // 128 blocks a vector and with this rule: 256 vectors of 4096 doubles 5840 -> 5735 us, of
+  // 900 doubles with a sparse factor 3919 -> 3811.  FP32 (no gain from larger blocks:
+  // 4096 cells cost a 61 x 75 x 90 call 4 us) keeps 128 blocks from 260 000 cells on.
+  const size_t per = r64 ? 1024 : 2048;
+  const int nblk = (int)((n + per - 1) / per < (size_t)kResidBlocks ? (n + per - 1) / per : (size_t)kResidBlocks);
+  dim3 grd(nblk, nvec);
   if (r64) k_dots3_partial<double><<<grd, 256, 0, s>>>((const double*)r, (const double*)t, n, (Dots<double>*)part);
   else k_dots3_partial<float><<<grd, 256, 0, s>>>((const float*)r, (const float*)t, n, (Dots<double>*)part);
-  k_dots3_final<<<nvec, 256, 0, s>>>((const Dots<double>*)part, kResidBlocks, out);
+  k_dots3_final<<<nvec, 256, 0, s>>>((const Dots<double>*)part, nblk, out);
   return cudaGetLastError();
 }
 
