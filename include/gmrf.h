@@ -30,7 +30,8 @@
  * element i of vector s is at [s*n + i] ("[nvec][n]" layout).
  *
  * Memory: every pointer argument may be host memory or device memory of the
- * current device (detected with cudaPointerGetAttributes).  The caller keeps
+ * current device (detected with cudaPointerGetAttributes), aligned for its
+ * element type; no wider alignment is asked for.  The caller keeps
  * ownership of everything it passes; the library copies kappa2 during
  * gmrf_create and owns its own workspaces (Lanczos basis, scalars,
  * transform tables), which gmrf_destroy frees.

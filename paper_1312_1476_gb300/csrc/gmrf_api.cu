@@ -1297,12 +1297,14 @@ int gmrf_apply(gmrf_problem* p, int32_t which, int64_t nvec, const void* v, void
   const bool vd = is_device_ptr(v), yd = is_device_ptr(y);
   const void* vin = v;
   void* yout = y;
-  if (!vd) {
+  // the kernels of A v move whole vectors: an array that lies at an odd element goes through a copy
+  auto direct = [&](const void* a) { return which != 1 || p->sp || precond_rows_aligned(p->pre, a); };
+  if (!vd || !direct(v)) {
     CKR(ensure(p->stage, bytes, p->ws));
-    CK(cudaMemcpyAsync(p->stage.p, v, bytes, cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(p->stage.p, v, bytes, vd ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     vin = p->stage.p;
   }
-  if (!yd) {
+  if (!yd || !direct(y)) {
     CKR(ensure(p->stage2, bytes, p->ws));
     yout = p->stage2.p;
   }
@@ -1327,7 +1329,7 @@ int gmrf_apply(gmrf_problem* p, int32_t which, int64_t nvec, const void* v, void
               [&] { return launch_precond_apply(p->pre, p->g, p->fp64, PRE_INV_SQRT, vin, yout, (int)nvec, s,
                                                  1.0 / std::sqrt(p->tau)); }));
   }
-  if (!yd) CK(cudaMemcpyAsync(y, yout, bytes, cudaMemcpyDeviceToHost, s));
+  if (yout != y) CK(cudaMemcpyAsync(y, yout, bytes, yd ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   trace_collect();
   CKR(leave(p));

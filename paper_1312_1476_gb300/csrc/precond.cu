@@ -1117,6 +1117,10 @@ cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int
   return run_apply<float, GMRF_PREC_MIRROR>(t, g, in, out, nvec, s, scale);
 }
 
+bool precond_rows_aligned(const PrecondTables& t, const void* v) {
+  return !t.line || line::row_aligned(t.kind, t.fp64 ? 8 : 4, v);
+}
+
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec) {
   return (size_t)nvec * t.ny * (t.nx + 2) * (t.fp64 ? 8 : 4);
 }

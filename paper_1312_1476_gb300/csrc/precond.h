@@ -81,7 +81,9 @@ cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec);
 cudaError_t launch_precond_apply_with(PrecondTables& t, const Grid& g, bool fp64, const void* in, void* out, int nvec,
                                       void* S, cudaStream_t s, double scale = 1.0);
-// y = A v for nvec vectors.
+// y = A v for nvec vectors, v and y aligned as precond_rows_aligned asks
+// (launch_precond_apply takes any element-aligned array).
+bool precond_rows_aligned(const PrecondTables& t, const void* v);
 cudaError_t launch_precond_operator(PrecondTables& t, const Grid& g, bool fp64, const void* kappa2,
                                     double kappa2_const, const void* v, void* y, int nvec, cudaStream_t s);
 

@@ -302,6 +302,24 @@ __device__ __forceinline__ void store_row(const typename C2<R>::T (&p)[8], R* __
       st4(dst + 4 * (t + T * r), p[2 * r].x, p[2 * r].y, p[2 * r + 1].x, p[2 * r + 1].y);
   }
 }
+// The same by element, for a caller's array that is not aligned for the vector accesses.
+template <typename R, int KIND, int T>
+__device__ __forceinline__ void load_row_elem(typename C2<R>::T (&p)[8], const R* __restrict__ src, int t) {
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const R* q = src + pair_at<KIND, T>(t, r);
+    p[r] = mk<typename C2<R>::T>(q[0], q[1]);
+  }
+}
+template <typename R, int KIND, int T>
+__device__ __forceinline__ void store_row_elem(const typename C2<R>::T (&p)[8], R* __restrict__ dst, int t) {
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    R* q = dst + pair_at<KIND, T>(t, r);
+    q[0] = p[r].x;
+    q[1] = p[r].y;
+  }
+}
 template <typename R, int KIND, int T>
 __device__ __forceinline__ void store_row_bf16(const typename C2<R>::T (&p)[8], __nv_bfloat16* dst, int t) {
   if constexpr (KIND == GMRF_PREC_CIRCULANT) {
@@ -549,7 +567,9 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
 
   if constexpr (MODE == L_FWD) {
     if (!step) {
-      load_row<R, KIND, T>(p, a.in + (size_t)s * n + ro, t);
+      const R* src = a.in + (size_t)s * n + ro;
+      if (a.in_elem) load_row_elem<R, KIND, T>(p, src, t);
+      else load_row<R, KIND, T>(p, src, t);
     } else {
       load_row<R, KIND, T>(p, ((j & 1) ? a.W1 : a.W0) + (size_t)s * n + ro, t);
       const R inv_b = (R)a.st[s].vscale;
@@ -593,7 +613,11 @@ __global__ void __launch_bounds__(block_threads(NX)) k_line_row(Args<R> a) {
   if constexpr (MODE == L_INV) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) p[r] = mk<C>(p[r].x * a.scale, p[r].y * a.scale);
-    if (live) store_row<R, KIND, T>(p, a.out + (size_t)s * n + ro, t);
+    if (live) {
+      R* dst = a.out + (size_t)s * n + ro;
+      if (a.out_elem) store_row_elem<R, KIND, T>(p, dst, t);
+      else store_row<R, KIND, T>(p, dst, t);
+    }
     return;
   }
   if constexpr (MODE == L_MIDW) {
@@ -954,17 +978,20 @@ cudaError_t step_k(const Args<R>& a, int nvec, cudaStream_t s) {
   return row_launch<R, KIND, L_LAST>(a, nvec, s, KC_PRE_ROW_LAST);
 }
 
-// out = scale B_bar^{-1} in
+// out = scale B_bar^{-1} in; in and out are the caller's own arrays and may lie at any element
 template <typename R, int KIND>
-cudaError_t apply_k(const Args<R>& a, int nvec, cudaStream_t s) {
+cudaError_t apply_k(Args<R> a, int nvec, cudaStream_t s) {
+  a.in_elem = !row_aligned(KIND, sizeof(R), a.in);
+  a.out_elem = !row_aligned(KIND, sizeof(R), a.out);
   LINE_CK((row_launch<R, KIND, L_FWD>(a, nvec, s, KC_PRE_APPLY)));
   LINE_CK((col_launch<R, KIND>(a, nvec, 0, s, KC_PRE_APPLY)));
   return row_launch<R, KIND, L_INV>(a, nvec, s, KC_PRE_APPLY);
 }
 
-// out = A in
+// out = A in; in and out aligned for whole vectors (row_aligned)
 template <typename R, int KIND>
 cudaError_t operator_k(const Args<R>& a, int nvec, cudaStream_t s) {
+  if (!row_aligned(KIND, sizeof(R), a.in) || !row_aligned(KIND, sizeof(R), a.out)) return cudaErrorMisalignedAddress;
   LINE_CK((first_passes<R, KIND>(a, nvec, 0, s, true)));
   return row_launch<R, KIND, L_LAST>(a, nvec, s, KC_PRE_APPLY);
 }

@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
+#include <cstdint>
 #include <vector>
 
 #include "precond.h"
@@ -49,6 +51,7 @@ struct Args {
   const R* in;
   R* out;
   R scale;              // of out (L_INV)
+  bool in_elem, out_elem;  // in / out not aligned for vectors (L_FWD, L_INV)
   const float* kappa2;
   R kappa2_const;
   size_t n;
@@ -64,6 +67,14 @@ struct Args {
   Dots<R>* partials;
   unsigned* counters;
 };
+
+// Whether the rows of an array can be taken by the widest accesses of load_row and
+// store_row: four reals for MIRROR, a complex pair for CIRCULANT, 16 bytes at most
+// (a row is a multiple of them, so the base decides).
+inline bool row_aligned(int kind, size_t es, const void* p) {
+  const size_t b = kind == GMRF_PREC_MIRROR || es == 8 ? 16 : 8;
+  return (reinterpret_cast<uintptr_t>(p) & (b - 1)) == 0;
+}
 
 // Host tables of a grid: FFT twiddles, pair factors and column coefficients.
 struct HostTables {
