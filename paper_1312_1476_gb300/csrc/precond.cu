@@ -1118,7 +1118,7 @@ cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int
 }
 
 bool precond_rows_aligned(const PrecondTables& t, const void* v) {
-  return !t.line || line::row_aligned(t.kind, t.fp64 ? 8 : 4, v);
+  return !(t.line || t.fast) || row_aligned(t.kind, t.fp64 ? 8 : 4, v);
 }
 
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec) {

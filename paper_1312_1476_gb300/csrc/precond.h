@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 #include <stddef.h>
+#include <stdint.h>
 
 #include "internal.h"
 
@@ -81,6 +82,13 @@ cudaError_t launch_precond_apply(PrecondTables& t, const Grid& g, bool fp64, int
 size_t precond_apply_scratch_bytes(const PrecondTables& t, int nvec);
 cudaError_t launch_precond_apply_with(PrecondTables& t, const Grid& g, bool fp64, const void* in, void* out, int nvec,
                                       void* S, cudaStream_t s, double scale = 1.0);
+// Whether the kernels that hold rows in registers can take an array's rows by their
+// widest accesses: four reals for MIRROR, a complex pair for CIRCULANT, 16 bytes at
+// most (a row is a multiple of them, so the base decides).
+inline bool row_aligned(int kind, size_t es, const void* p) {
+  const size_t b = kind == GMRF_PREC_MIRROR || es == 8 ? 16 : 8;
+  return (reinterpret_cast<uintptr_t>(p) & (b - 1)) == 0;
+}
 // y = A v for nvec vectors, v and y aligned as precond_rows_aligned asks
 // (launch_precond_apply takes any element-aligned array).
 bool precond_rows_aligned(const PrecondTables& t, const void* v);

@@ -337,6 +337,26 @@ __device__ __forceinline__ void store_row(const float2* p, float* __restrict__ d
       *reinterpret_cast<float4*>(dst + 4 * (lane + 32 * r)) = make_float4(p[2 * r].x, p[2 * r].y, p[2 * r + 1].x, p[2 * r + 1].y);
   }
 }
+// The same by element, for a caller's array that is not aligned for the vector accesses.
+template <int KIND, int E>
+__device__ __forceinline__ void load_row_elem(float2* p, const float* __restrict__ src) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    const float* q = src + pair_off<KIND, E>(lane, r);
+    p[r] = f2(q[0], q[1]);
+  }
+}
+template <int KIND, int E>
+__device__ __forceinline__ void store_row_elem(const float2* p, float* __restrict__ dst) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < E; ++r) {
+    float* q = dst + pair_off<KIND, E>(lane, r);
+    q[0] = p[r].x;
+    q[1] = p[r].y;
+  }
+}
 template <int KIND, int E>
 __device__ __forceinline__ void store_row_bf16(const float2* p, __nv_bfloat16* dst) {
   const int lane = threadIdx.x & 31;
@@ -665,7 +685,8 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const size_t ro = (size_t)(y0 + tr0 + g) * NX;
-      load_row<KIND, E>(p + g * E, Win + ro);
+      if (a.in_elem) load_row_elem<KIND, E>(p + g * E, Win + ro);  // plain applies only
+      else load_row<KIND, E>(p + g * E, Win + ro);
       if (Vp) load_row<KIND, E>(qv + g * E, Vp + ro);
     }
     stage_tables();
@@ -716,7 +737,11 @@ __global__ void __launch_bounds__(32 * (rows_per_block<KIND, LOGL>() / lpw<LOGL>
   if (MODE != R_MIDG) rows_inverse<KIND, LOGL>(a, p, sm, tile, tr0, twx, ptx);
   if (MODE == R_INV) {
 #pragma unroll
-    for (int g = 0; g < G; ++g) store_row<KIND, E>(p + g * E, a.out + (size_t)s * n + (size_t)(y0 + tr0 + g) * NX);
+    for (int g = 0; g < G; ++g) {
+      float* dst = a.out + (size_t)s * n + (size_t)(y0 + tr0 + g) * NX;
+      if (a.out_elem) store_row_elem<KIND, E>(p + g * E, dst);
+      else store_row<KIND, E>(p + g * E, dst);
+    }
     return;
   }
   if (MODE == R_MIDW) {
@@ -1113,18 +1138,22 @@ cudaError_t step_k(const Args& a, int nvec, cudaStream_t s) {
   return cudaSuccess;
 }
 
-// out = B_bar^{-p/2} in
+// out = B_bar^{-p/2} in; in and out are the caller's own arrays and may lie at any element
 template <int KIND>
-cudaError_t apply_k(const Args& a, int nvec, cudaStream_t s) {
+cudaError_t apply_k(Args a, int nvec, cudaStream_t s) {
+  a.in_elem = !row_aligned(KIND, sizeof(float), a.in);
+  a.out_elem = !row_aligned(KIND, sizeof(float), a.out);
   FAST_CK((row_launch<KIND, R_FWD>(a, nvec, s, KC_PRE_APPLY)));
   FAST_CK((col_launch<KIND>(a, nvec, 0, s, KC_PRE_APPLY)));
   FAST_CK((row_launch<KIND, R_INV>(a, nvec, s, KC_PRE_APPLY)));
   return cudaSuccess;
 }
 
-// out = A in
+// out = A in; in and out aligned for whole vectors (row_aligned)
 template <int KIND>
 cudaError_t operator_k(const Args& a, int nvec, cudaStream_t s) {
+  if (!row_aligned(KIND, sizeof(float), a.in) || !row_aligned(KIND, sizeof(float), a.out))
+    return cudaErrorMisalignedAddress;
   FAST_CK((row_launch<KIND, R_FWD>(a, nvec, s, KC_PRE_APPLY)));
   FAST_CK((col_launch<KIND>(a, nvec, 0, s, KC_PRE_APPLY)));
   if (host_edge_terms(KIND, a.bc)) {

@@ -28,6 +28,7 @@ struct Args {
   float* Wg;           // w when the y-boundary terms need a separate pass
   const float* in;
   float* out;
+  bool in_elem, out_elem;  // in / out of a plain apply not aligned for vectors
   const float* kappa2;
   float kappa2_const;
   size_t n;

@@ -5,8 +5,6 @@
 
 #include <cuda_runtime.h>
 
-#include <cstddef>
-#include <cstdint>
 #include <vector>
 
 #include "precond.h"
@@ -67,14 +65,6 @@ struct Args {
   Dots<R>* partials;
   unsigned* counters;
 };
-
-// Whether the rows of an array can be taken by the widest accesses of load_row and
-// store_row: four reals for MIRROR, a complex pair for CIRCULANT, 16 bytes at most
-// (a row is a multiple of them, so the base decides).
-inline bool row_aligned(int kind, size_t es, const void* p) {
-  const size_t b = kind == GMRF_PREC_MIRROR || es == 8 ? 16 : 8;
-  return (reinterpret_cast<uintptr_t>(p) & (b - 1)) == 0;
-}
 
 // Host tables of a grid: FFT twiddles, pair factors and column coefficients.
 struct HostTables {

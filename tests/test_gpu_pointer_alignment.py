@@ -59,6 +59,17 @@ def test_squared_operator_on_shifted_arrays(shape, precision, shift, kind, bc):
         _same_calls(p, shape[0] * shape[1], torch.float64 if f64 else torch.float32, shift, 1e-9 if f64 else 1e-5)
 
 
+@pytest.mark.parametrize("kind,bc", [("mirror", "neumann"), ("circulant", "periodic"), ("mirror", "dirichlet")])
+@pytest.mark.parametrize("shift", [1, 2])
+@pytest.mark.parametrize("shape", [(128, 128), (128, 1024), (256, 2048)], ids=lambda s: "%dx%d" % s)
+def test_shifted_laplacian_on_shifted_arrays(shape, shift, kind, bc):
+    from paper_1312_1476_gb300 import gmrf
+    g = torch.Generator(device="cuda").manual_seed(2)
+    k2 = torch.rand(shape, generator=g, device="cuda") + 0.5
+    with gmrf.Problem(shape, bc, "shifted_laplacian", kappa2=k2, tau=0.7, precond=kind) as p:
+        _same_calls(p, shape[0] * shape[1], torch.float32, shift, 1e-5)
+
+
 def test_server_writes_shifted_arrays():
     from paper_1312_1476_gb300 import gmrf
     shape, n = (64, 64), 4096
