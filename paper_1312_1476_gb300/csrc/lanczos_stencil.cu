@@ -425,11 +425,12 @@ __global__ void __launch_bounds__(NT3) k_stencil3d(StencilArgs<T> a) {
     finish_step<T>(a.P, j, s, a.partials, nblk, a.st, a.alpha, a.beta, a.alpha_f, a.beta2_f, red, s_int, s_flt);
 }
 
-// cells per thread along x for the 3-D kernel
-int vx3(const Grid& g, bool fp64) {
-  if (!fp64 && g.nx % 4 == 0 && g.nx >= 128) return 4;
-  if (g.nx % 2 == 0 && g.nx >= 64) return 2;
-  return 1;
+// cells per thread along x for the 3-D kernel: one where a caller's array (apply
+// mode) is not aligned for accesses of more
+int vx3(const Grid& g, bool fp64, const void* win, const void* wout) {
+  const int vx = !fp64 && g.nx % 4 == 0 && g.nx >= 128 ? 4 : (g.nx % 2 == 0 && g.nx >= 64 ? 2 : 1);
+  const uintptr_t at = (uintptr_t)win | (uintptr_t)wout;
+  return at % (vx * (fp64 ? 8 : 4)) == 0 ? vx : 1;
 }
 
 int nz_chunks(const Grid& g, int vx) {
@@ -456,7 +457,7 @@ cudaError_t dispatch(const Grid& g, StencilArgs<T> a, int nvec, cudaStream_t s, 
         return launch_stencil3d_tma(g, a, nvec, STEP, s);
     }
     if (stencil3d_flat_eligible(g)) return launch_stencil3d_flat<T>(g, a, nvec, STEP, s);
-    const int vx = vx3(g, sizeof(T) == 8);
+    const int vx = vx3(g, sizeof(T) == 8, STEP ? nullptr : a.Win, STEP ? nullptr : a.Wout);
     a.nzc = nz_chunks(g, vx);
     blk = dim3(TX, TY3);
     grd = dim3((g.nx + TX * vx - 1) / (TX * vx), (g.ny + TY3 - 1) / TY3, nvec * a.nzc);

@@ -70,6 +70,26 @@ def test_shifted_laplacian_on_shifted_arrays(shape, shift, kind, bc):
         _same_calls(p, shape[0] * shape[1], torch.float32, shift, 1e-5)
 
 
+@pytest.mark.parametrize("bc", ["periodic", "neumann", "dirichlet"])
+@pytest.mark.parametrize("precision,shift", [("fp32", 1), ("fp32", 2), ("fp64", 1)])
+@pytest.mark.parametrize("nx", [516, 518, 1024])
+def test_wide_3d_product_on_shifted_arrays(nx, precision, shift, bc):
+    from paper_1312_1476_gb300 import gmrf
+    shape, n = (5, 9, nx), 45 * nx
+    dtype = torch.float64 if precision == "fp64" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(4)
+    k2 = torch.rand(shape, generator=g, device="cuda") + 0.5
+    v = _randn(2 * n, dtype, 6)
+    with gmrf.Problem(shape, bc, "shifted_laplacian", kappa2=k2, precision=precision) as p:
+        want = torch.empty_like(v)
+        p.apply(0, v, want, nvec=2)
+        for a, y in ((_shifted(v, shift), torch.empty_like(v)), (v, _shifted(v, shift)),
+                     (_shifted(v, shift), _shifted(v, shift))):
+            p.apply(0, a, y.fill_(float("nan")), nvec=2)
+            # one cell a thread instead of two or four: up to eleven roundings of terms of at most 8 max |v|
+            assert (y - want).abs().max() <= 12 * 13.5 * torch.finfo(dtype).eps * v.abs().max()
+
+
 def test_server_writes_shifted_arrays():
     from paper_1312_1476_gb300 import gmrf
     shape, n = (64, 64), 4096
