@@ -32,10 +32,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
-#include <atomic>
 #include <vector>
 
 #include "fft.cuh"
+#include "per_device.h"
 #include "precond.h"
 #include "precond_fast.h"
 #include "precond_line.h"
@@ -689,38 +689,40 @@ line::Args<R> line_args(const PrecondTables& t, const Grid& g, const void* kappa
 }
 
 int smem_optin() {
-  static const int v = [] {  // thread-safe one-time initialisation
-    int dev = 0, r = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&r, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-      cudaGetLastError();
-      r = 48 * 1024;
-    }
-    return r;
-  }();
-  return v;
+  static PerDevice optin;
+  int v = 0;
+  const cudaError_t e = optin.get(
+      [](int* r) {
+        int dev = 0;
+        const cudaError_t e = cudaGetDevice(&dev);
+        return e != cudaSuccess ? e : cudaDeviceGetAttribute(r, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+      },
+      &v);
+  if (e == cudaSuccess) return v;
+  cudaGetLastError();
+  return 48 * 1024;
 }
 
-// Raise the dynamic shared memory limit of a kernel once per process.
+// Raise the dynamic shared memory limit of a kernel once per device.
 template <typename K>
-cudaError_t allow_smem(K* k, std::atomic<bool>& done) {
-  if (done.load(std::memory_order_acquire)) return cudaSuccess;
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, k);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - (int)fa.sharedSizeBytes);
-  if (e == cudaSuccess) done.store(true, std::memory_order_release);
-  return e;
+cudaError_t allow_smem(K* k, PerDevice& done) {
+  return done.get([&](int* v) {
+    *v = 1;
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, k);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - (int)fa.sharedSizeBytes);
+  });
 }
 
 template <typename R, int KIND, int MODE>
 cudaError_t row_attr() {
-  static std::atomic<bool> done{false};
+  static PerDevice done;
   return allow_smem(k_prow<R, KIND, MODE>, done);
 }
 template <typename R, int KIND>
 cudaError_t col_attr() {
-  static std::atomic<bool> done{false};
+  static PerDevice done;
   return allow_smem(k_pcol<R, KIND>, done);
 }
 

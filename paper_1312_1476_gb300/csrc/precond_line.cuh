@@ -39,9 +39,9 @@
 
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <utility>
 
+#include "per_device.h"
 #include "precond_line.h"
 #include "trace.h"
 
@@ -887,11 +887,8 @@ template <typename R, int KIND, int NX, int MODE>
 cudaError_t row_launch_t(const Args<R>& a, int nvec, cudaStream_t s, int kc) {
   constexpr size_t sm = row_smem<R, NX>();
   if constexpr (sm > 40 * 1024) {
-    static std::atomic<bool> attr{false};  // several host threads may launch at once
-    if (!attr.load(std::memory_order_acquire)) {
-      LINE_CK(cudaFuncSetAttribute(k_line_row<R, KIND, NX, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-      attr.store(true, std::memory_order_release);
-    }
+    static PerDevice attr;
+    LINE_CK(set_attribute(attr, k_line_row<R, KIND, NX, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   }
   dim3 grd((a.ny + block_rows(NX) - 1) / block_rows(NX), nvec);
   trace_begin(kc, s);

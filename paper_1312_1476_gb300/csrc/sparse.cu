@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "per_device.h"
 
 namespace gmrf {
 
@@ -497,12 +498,19 @@ size_t raise_smem(K kernel) {
   return (size_t)avail;
 }
 
-// Done once per precision, at problem creation (outside any stream capture):
-// the dynamic shared memory both kernels may use.
+// Done once per precision and device, at problem creation (outside any stream
+// capture): the dynamic shared memory both kernels may use, 0 on error.
 template <typename T>
 size_t kernels_smem_limit() {
-  static const size_t lim = std::min(raise_smem(k_sparse_step<T>), raise_smem(k_sparse_ops<T>));
-  return lim;
+  static PerDevice limit;
+  int lim = 0;
+  const cudaError_t e = limit.get(
+      [](int* v) {
+        *v = (int)std::min(raise_smem(k_sparse_step<T>), raise_smem(k_sparse_ops<T>));
+        return *v > 0 ? cudaSuccess : cudaErrorInvalidValue;
+      },
+      &lim);
+  return e == cudaSuccess ? (size_t)lim : 0;
 }
 
 template <typename T>

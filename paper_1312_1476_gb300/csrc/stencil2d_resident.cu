@@ -30,10 +30,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 
 #include "internal.h"
+#include "per_device.h"
 #include "stencil_args.h"
 
 namespace gmrf {
@@ -239,12 +239,9 @@ int tiles_of(const Grid& g) {
 
 template <typename T, int BC>
 cudaError_t launch(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps, cudaStream_t s) {
-  static std::atomic<bool> attr{false};  // several host threads may launch at once
-  if (!attr.load(std::memory_order_acquire)) {
-    const cudaError_t e = cudaFuncSetAttribute(k_resident2d<T, BC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attr.store(true, std::memory_order_release);
-  }
+  static PerDevice attr;
+  const cudaError_t e = set_attribute(attr, k_resident2d<T, BC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
   const int tiles = tiles_of<T>(g);
   int ncl = 1;
   while (ncl < kMaxCluster && ncl < tiles) ncl *= 2;

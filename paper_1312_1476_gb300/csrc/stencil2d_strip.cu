@@ -22,10 +22,10 @@
 // a vector do not depend on the rest of its batch.
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <cstdint>
 
 #include "internal.h"
+#include "per_device.h"
 #include "stencil_args.h"
 
 namespace gmrf {
@@ -458,13 +458,10 @@ int strip_ychunk(const Grid& g) {
 template <typename T, int OP, int BC, bool STEP, bool AL>
 cudaError_t launch_al(dim3 grd, const StencilArgs<T>& a, int yc, cudaStream_t s) {
   constexpr size_t sm = strip_smem_bytes<T, OP, STEP, AL>();
-  static std::atomic<bool> attr{false};  // several host threads may launch at once
-  if (!attr.load(std::memory_order_acquire)) {
-    cudaError_t e = cudaFuncSetAttribute(k_stencil2d_strip<T, OP, BC, STEP, AL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    attr.store(true, std::memory_order_release);
-  }
+  static PerDevice attr;
+  const cudaError_t e = set_attribute(attr, k_stencil2d_strip<T, OP, BC, STEP, AL>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
   k_stencil2d_strip<T, OP, BC, STEP, AL><<<grd, SNT, sm, s>>>(a, yc);
   return cudaGetLastError();
 }

@@ -30,9 +30,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "internal.h"
+#include "per_device.h"
 #include "stencil_args.h"
 
 namespace gmrf {
@@ -330,14 +330,11 @@ Flat flat_plan(const Grid& g) {
 
 template <typename T, int BC, bool STEP, int FE>
 cudaError_t flat_launch_e(const Grid& g, const Flat& f, const StencilArgs<T>& a, int nvec, cudaStream_t s) {
-  static std::atomic<bool> attr{false};  // several host threads may launch at once
-  if (!attr.load(std::memory_order_acquire)) {
-    const cudaError_t e = cudaFuncSetAttribute(k_stencil3d_flat<T, BC, STEP, FE>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)(FSTAGES * flat_stage<T>(FNT * FE, FH * FNT / 2)));
-    if (e != cudaSuccess) return e;
-    attr.store(true, std::memory_order_release);
-  }
+  static PerDevice attr;
+  const cudaError_t e = set_attribute(attr, k_stencil3d_flat<T, BC, STEP, FE>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(FSTAGES * flat_stage<T>(FNT * FE, FH * FNT / 2)));
+  if (e != cudaSuccess) return e;
   k_stencil3d_flat<T, BC, STEP, FE><<<dim3(f.blocks, nvec), FNT, FSTAGES * flat_stage<T>(FNT * FE, g.nx), s>>>(
       a, f.nrange, f.zper);
   return cudaGetLastError();

@@ -27,6 +27,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "per_device.h"
 #include "stencil_args.h"
 #include "tma.cuh"
 
@@ -346,20 +347,20 @@ Items make_items(const Grid& g, int nvec) {
 template <int BC, bool STEP>
 cudaError_t launch_bc(const StencilArgs<float>& a, const Maps& maps, const Items& it, cudaStream_t s) {
   auto k = k_stencil3d_tma<BC, STEP>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  static int resident = 0;
-  std::call_once(once, [&] {
-    attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-    int per_sm = 0, dev = 0, nsm = 0;
-    if (attr_err == cudaSuccess) attr_err = cudaGetDevice(&dev);
-    if (attr_err == cudaSuccess) attr_err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (attr_err == cudaSuccess)
-      attr_err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, kSmemBytes);
-    resident = per_sm * nsm;
-    if (attr_err == cudaSuccess && resident < 1) attr_err = cudaErrorInvalidConfiguration;
-  });
-  if (attr_err != cudaSuccess) return attr_err;
+  static PerDevice blocks;
+  int resident = 0;
+  const cudaError_t err = blocks.get(
+      [&](int* v) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        int per_sm = 0, dev = 0, nsm = 0;
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, kSmemBytes);
+        *v = per_sm * nsm;
+        return e == cudaSuccess && *v < 1 ? cudaErrorInvalidConfiguration : e;
+      },
+      &resident);
+  if (err != cudaSuccess) return err;
   const int grid = it.total < resident ? it.total : resident;
   if (grid < 1) return cudaSuccess;
   k<<<grid, dim3(32, BY), kSmemBytes, s>>>(a, maps, it);
