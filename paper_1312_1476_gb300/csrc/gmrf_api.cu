@@ -723,6 +723,7 @@ int gmrf_create(const gmrf_desc* d, void* stream, gmrf_problem** out) {
     delete p;
     return GMRF_ERR_CUDA;
   }
+  if (p->precond == GMRF_PREC_NONE) p->g.clusters = stencil2d_resident_fits(p->g, p->fp64);
   auto fail = [&](int code) {
     gmrf_destroy(p);
     return code;

@@ -237,28 +237,58 @@ int tiles_of(const Grid& g) {
   return ((g.nx + kTileX - 1) / kTileX) * ((g.ny + tile2d_y<T>() - 1) / tile2d_y<T>());
 }
 
+// the launch of nvec vectors; returns the tiles of a block
 template <typename T, int BC>
-cudaError_t launch(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps, cudaStream_t s) {
+cudaError_t config(const Grid& g, int nvec, cudaLaunchConfig_t& c, cudaLaunchAttribute& at, int& tpb) {
   static PerDevice attr;
   const cudaError_t e = set_attribute(attr, k_resident2d<T, BC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   const int tiles = tiles_of<T>(g);
   int ncl = 1;
   while (ncl < kMaxCluster && ncl < tiles) ncl *= 2;
-  const int tpb = (tiles + ncl - 1) / ncl;
-  cudaLaunchConfig_t c = {};
+  tpb = (tiles + ncl - 1) / ncl;
+  c = {};
   c.gridDim = dim3(ncl, nvec);
   c.blockDim = dim3(tpb * tile2d_threads<T>());
   c.dynamicSmemBytes = ((size_t)tpb * kTileX * tile2d_y<T>() + 1) * sizeof(T);
-  c.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = ncl;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  c.attrs = at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ncl;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  c.attrs = &at;
   c.numAttrs = 1;
+  return cudaSuccess;
+}
+
+template <typename T, int BC>
+cudaError_t launch(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps, cudaStream_t s) {
+  cudaLaunchConfig_t c;
+  cudaLaunchAttribute at;
+  int tpb = 0;
+  const cudaError_t e = config<T, BC>(g, nvec, c, at, tpb);
+  if (e != cudaSuccess) return e;
+  c.stream = s;
   return cudaLaunchKernelEx(&c, k_resident2d<T, BC>, a, nsteps, tpb);
+}
+
+template <typename T, int BC>
+bool fits(const Grid& g) {
+  cudaLaunchConfig_t c;
+  cudaLaunchAttribute at;
+  int tpb = 0, n = 0;
+  if (config<T, BC>(g, 1, c, at, tpb) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, k_resident2d<T, BC>, &c) == cudaSuccess)
+    return n > 0;
+  cudaGetLastError();
+  return false;
+}
+template <typename T>
+bool fits(const Grid& g) {
+  switch (g.bc) {
+    case GMRF_BC_PERIODIC: return fits<T, GMRF_BC_PERIODIC>(g);
+    case GMRF_BC_NEUMANN: return fits<T, GMRF_BC_NEUMANN>(g);
+    default: return fits<T, GMRF_BC_DIRICHLET>(g);
+  }
 }
 
 }  // namespace
@@ -271,7 +301,7 @@ cudaError_t launch(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps,
 // More than a tile a block: FP64 91 x 77 (36 tiles) 4 vectors 1176 and 1245, 8 1552 and
 // 1440, 100 x 100 (52) one vector 1311 and 1221; FP32 91 x 77 (18) 8 vectors 647 and
 // 833, 16 1360 and 1275, 190 x 150 (60) 4 vectors 677 and 860.
-bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec) {
+static bool takes(const Grid& g, bool fp64, int nvec) {
   if (g.dim != 2 || g.op != GMRF_OP_SHIFTED_LAPLACIAN || stencil2d_strip_eligible(g, fp64)) return false;
   if (g.n > (size_t)kMaxTiles * 512) return false;
   const int tiles = fp64 ? tiles_of<double>(g) : tiles_of<float>(g);
@@ -279,6 +309,10 @@ bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec) {
   if (tiles <= kMaxCluster) return all <= (fp64 ? 5 : 2) * 152;
   return tiles <= (fp64 ? 3 * kMaxCluster : kMaxTiles) && all <= (fp64 ? 152 : 256);
 }
+bool stencil2d_resident_fits(const Grid& g, bool fp64) {
+  return takes(g, fp64, 1) && (fp64 ? fits<double>(g) : fits<float>(g));
+}
+bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec) { return g.clusters && takes(g, fp64, nvec); }
 
 template <typename T>
 cudaError_t launch_stencil2d_resident(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps, cudaStream_t s) {
