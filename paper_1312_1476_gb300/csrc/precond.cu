@@ -928,6 +928,18 @@ int upload_tables(PrecondTables& t, cudaStream_t s, std::vector<double>& lx64, s
     if (cudaMemcpyAsync(*dst, src, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return -1;
     return 0;
   };
+  // the line kernels have their own tables and read none of the others'
+  if (t.line) {
+    line::HostTables lt;
+    line::host_tables(t.kind, t.nx, t.ny, t.kbar2, lt);
+    const std::vector<R> ltw(lt.tw.begin(), lt.tw.end()), lpair(lt.pair.begin(), lt.pair.end()),
+        lcol(lt.col.begin(), lt.col.end());
+    if (up(&t.ltw, ltw.data(), ltw.size() * sizeof(R)) || up(&t.lpair, lpair.data(), lpair.size() * sizeof(R)) ||
+        up(&t.lcol, lcol.data(), lcol.size() * sizeof(R)))
+      return -1;
+    // host vectors must outlive the async copies
+    return cudaStreamSynchronize(s) == cudaSuccess ? 0 : -1;
+  }
   std::vector<R> lxr(lx64.begin(), lx64.end()), lyr(ly64.begin(), ly64.end());
   auto tw = [&](int N, std::vector<C>& out) {
     out.resize(N);
@@ -986,18 +998,7 @@ int upload_tables(PrecondTables& t, cudaStream_t s, std::vector<double>& lx64, s
     if (up(&t.pairx, prx.data(), prx.size() * sizeof(R)) || up(&t.pairy, pry.data(), pry.size() * sizeof(R)))
       return -1;
   }
-  line::HostTables lt;
-  std::vector<R> ltw, lpair, lcol;
-  if (t.line) {
-    line::host_tables(t.kind, t.nx, t.ny, t.kbar2, lt);
-    ltw.assign(lt.tw.begin(), lt.tw.end());
-    lpair.assign(lt.pair.begin(), lt.pair.end());
-    lcol.assign(lt.col.begin(), lt.col.end());
-    if (up(&t.ltw, ltw.data(), ltw.size() * sizeof(R)) || up(&t.lpair, lpair.data(), lpair.size() * sizeof(R)) ||
-        up(&t.lcol, lcol.data(), lcol.size() * sizeof(R)))
-      return -1;
-  }
-  // host vectors must outlive the async copies
+  // as above
   return cudaStreamSynchronize(s) == cudaSuccess ? 0 : -1;
 }
 
@@ -1084,6 +1085,7 @@ int precond_blocks_per_vector(const PrecondTables& t) {
 
 int precond_prepare(PrecondTables& t, int nvec, cudaStream_t s) {
   if (ensure_ws(t, nvec, s)) return GMRF_ERR_OOM;
+  if (t.line || t.fast) return GMRF_OK;  // no generic kernel is launched
   cudaError_t e;
   if (t.fp64) e = t.kind == GMRF_PREC_CIRCULANT ? set_attrs<double, GMRF_PREC_CIRCULANT>()
                                                : set_attrs<double, GMRF_PREC_MIRROR>();
