@@ -28,6 +28,7 @@
 
 #include "internal.h"
 #include "per_device.h"
+#include "tri_schedule.h"
 
 namespace gmrf {
 
@@ -53,7 +54,7 @@ struct SparseOp {
 
 namespace {
 
-constexpr int kSpThreads = 256;
+constexpr int kSpThreads = kTriThreads;
 
 // ------------------------------------------------------------------ host: CSR
 struct HostCsr {
@@ -536,144 +537,6 @@ cudaError_t sparse_ops_t(const SparseOp& S, int mode, const void* in, void* out,
   return cudaGetLastError();
 }
 
-// Level of every row: forward (row i after the rows k < i it reads) or
-// backward (row i after the rows k > i it reads); rows grouped by level.
-void levels(int n, const std::vector<int>& ptr, const std::vector<int>& col, bool forward, std::vector<int>& rows,
-            std::vector<int>& lptr) {
-  std::vector<int> lev((size_t)n, 0);
-  int nlev = 0;
-  for (int t = 0; t < n; ++t) {
-    const int i = forward ? t : n - 1 - t;
-    int l = 0;
-    for (int e = ptr[(size_t)i]; e < ptr[(size_t)i + 1]; ++e) l = std::max(l, lev[(size_t)col[(size_t)e]] + 1);
-    lev[(size_t)i] = l;
-    nlev = std::max(nlev, l + 1);
-  }
-  lptr.assign((size_t)nlev + 1, 0);
-  for (int i = 0; i < n; ++i) ++lptr[(size_t)lev[(size_t)i] + 1];
-  for (int l = 0; l < nlev; ++l) lptr[(size_t)l + 1] += lptr[(size_t)l];
-  rows.assign((size_t)n, 0);
-  std::vector<int> fill(lptr.begin(), lptr.end() - 1);
-  for (int i = 0; i < n; ++i) rows[(size_t)fill[(size_t)lev[(size_t)i]]++] = i;
-}
-
-// The schedule of one substitution.  Consecutive levels are merged into one:
-// with the rows B of the merged levels and the rows P before them,
-//   x_B = F_BB^{-1} b_B - F_BB^{-1} F_BP x_P,
-// so every row of B is a dot product over right-hand sides of B and results of
-// P, at the price of the fill that the small inverse brings.  A level costs a
-// chain of dependent operations and a barrier whatever it holds (about
-// kLevelCycles), an entry its share of the FP64 lanes and of the loads (kEntryCycles),
-// so the next level is merged while the entries it adds cost less than that.
-// Merged rows stay below kMergedRow entries.  The values are formed in FP64.
-// kEntryCycles and the six entries per lane are the best of a sweep on the
-// Figure 3 matrix, 256 samples, drop tolerance 1e-3 / 1e-5 / 1e-2 (FP64): 4.2 /
-// 6.4 / 12.5 ms a call at 3 cycles, 6.4 / 6.4 / 14.4 at 1.5, 7.9 / 7.3 / 19.4 at 14;
-// 10.7 / 29.1 / 26.3 ms level by level.  The factor with 1e-3 goes from 204 to 39
-// levels and from 13.4k to 29.5k entries.
-struct TriHost {
-  std::vector<int> rec, row, col;
-  std::vector<double> val;
-};
-constexpr double kLevelCycles = 500.0;
-constexpr double kEntryCycles = 3.0;
-constexpr int kMergedRow = 128;
-
-// rows in level order (lptr); ptr/col/val the off-diagonal entries of each row;
-// b and x the positions of the right-hand side and of the result in the shared arrays
-void tri_schedule(int n, const std::vector<int>& rows, const std::vector<int>& lptr, const std::vector<int>& ptr,
-                  const std::vector<int>& col, const std::vector<double>& val, const std::vector<double>& dg, int b0,
-                  int x0, TriHost& out) {
-  const int nlev = (int)lptr.size() - 1;
-  typedef std::vector<std::pair<int, double>> Expr;  // (position, coefficient)
-  std::vector<Expr> expr((size_t)n);  // of the rows of the merged level being built
-  std::vector<int> in_block((size_t)n, -1);
-  std::vector<double> acc((size_t)std::max(b0, x0) + n, 0.0);
-  std::vector<int> stamp(acc.size(), -1), used;
-  int block = 0, mark = 0;
-  auto row_expr = [&](int i, Expr& e) {
-    ++mark;
-    used.clear();
-    auto add = [&](int at, double w) {
-      if (stamp[(size_t)at] != mark) {
-        stamp[(size_t)at] = mark;
-        acc[(size_t)at] = 0.0;
-        used.push_back(at);
-      }
-      acc[(size_t)at] += w;
-    };
-    add(b0 + i, 1.0);
-    for (int q = ptr[(size_t)i]; q < ptr[(size_t)i + 1]; ++q) {
-      const int k = col[(size_t)q];
-      if (in_block[(size_t)k] == block)
-        for (const auto& t : expr[(size_t)k]) add(t.first, -val[(size_t)q] * t.second);
-      else
-        add(x0 + k, -val[(size_t)q]);
-    }
-    e.clear();
-    for (int at : used) e.emplace_back(at, acc[(size_t)at] / dg[(size_t)i]);
-  };
-  out = TriHost();
-  std::vector<Expr> cand;
-  for (int l = 0; l < nlev;) {
-    ++block;
-    std::vector<int> members;
-    int end = l;
-    for (; end < nlev; ++end) {
-      cand.clear();
-      double extra = 0.0;
-      size_t longest = 0;
-      for (int q = lptr[(size_t)end]; q < lptr[(size_t)end + 1]; ++q) {
-        const int i = rows[(size_t)q];
-        Expr e;
-        row_expr(i, e);
-        extra += (double)e.size() - (double)(ptr[(size_t)i + 1] - ptr[(size_t)i] + 1);
-        longest = std::max(longest, e.size());
-        cand.push_back(std::move(e));
-      }
-      if (end > l && (extra * kEntryCycles > kLevelCycles || longest > (size_t)kMergedRow)) break;
-      for (int q = lptr[(size_t)end]; q < lptr[(size_t)end + 1]; ++q) {
-        const int i = rows[(size_t)q];
-        expr[(size_t)i] = std::move(cand[(size_t)(q - lptr[(size_t)end])]);
-        in_block[(size_t)i] = block;
-        members.push_back(i);
-      }
-    }
-    l = end;
-    // rounds of the merged level: rows by length, about six entries per lane
-    std::stable_sort(members.begin(), members.end(),
-                     [&](int p, int q) { return expr[(size_t)p].size() > expr[(size_t)q].size(); });
-    double mean = 0.0;
-    for (int i : members) mean += (double)expr[(size_t)i].size();
-    mean /= (double)members.size();
-    int lg = 0;
-    while (lg < 5 && 6.0 * (1 << lg) < mean) ++lg;
-    const int per = kSpThreads >> lg;
-    for (size_t m0 = 0; m0 < members.size(); m0 += (size_t)per) {
-      const int cnt = (int)std::min((size_t)per, members.size() - m0);
-      const int lanes = ((cnt << lg) + 31) / 32 * 32;
-      const int slots = (int)((expr[(size_t)members[m0]].size() + (1u << lg) - 1) >> lg);
-      const size_t off = out.col.size();
-      const int rec[8] = {(int)off, slots, lanes, lg, (int)out.row.size(), cnt,
-                          m0 + (size_t)per >= members.size() ? 1 : 0, 0};
-      out.rec.insert(out.rec.end(), rec, rec + 8);
-      out.col.resize(off + (size_t)slots * lanes, -1);
-      out.val.resize(out.col.size(), 0.0);
-      for (int r = 0; r < cnt; ++r) {
-        const int i = members[m0 + (size_t)r];
-        out.row.push_back(i);
-        const Expr& e = expr[(size_t)i];
-        for (size_t t = 0; t < e.size(); ++t) {
-          const size_t at = off + (t >> lg) * (size_t)lanes + ((size_t)r << lg) + (t & ((1u << lg) - 1));
-          out.col[at] = e[t].first;
-          out.val[at] = e[t].second;
-        }
-      }
-    }
-    for (int i : members) Expr().swap(expr[(size_t)i]);
-  }
-}
-
 template <typename T>
 int upload(void** dst, const std::vector<double>& v, cudaStream_t s) {
   std::vector<T> h(v.begin(), v.end());
@@ -769,8 +632,8 @@ int sparse_create(SparseOp** out, const gmrf_sparse_desc* d, bool fp64, cudaStre
     // shared arrays of the kernels: 0 .. n - 1 the input of F^{-T}, n .. 2n - 1 the results, 2n .. 3n - 1 the input of F^{-1}
     TriHost th[2];
     try {
-      tri_schedule(n, rf, pf, lp, lc, lv, dg, 2 * n, n, th[0]);
-      tri_schedule(n, rb, pb, up, uc, uv, dg, 0, n, th[1]);
+      tri_schedule(n, rf, pf, lp, lc, lv, dg, true, 2 * n, n, th[0]);
+      tri_schedule(n, rb, pb, up, uc, uv, dg, false, 0, n, th[1]);
     } catch (const std::bad_alloc&) {
       return fail(GMRF_ERR_OOM);
     }
