@@ -638,7 +638,15 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
     } else {
       const double ud = u * dinv;
       energy += u * ud;
-      const double rr2 = (is_positive(b2) ? b2 : 0.0) * (ud * ud);  // (||r_m|| / ||z||)^2
+      // (||r_m|| / ||z||)^2, compared with tol^2 to save the square roots of a step that
+      // does not stop.  Both underflow for tolerances below 1e-154, so a stop is decided on
+      // the residual itself, formed from the factors where the square has lost digits
+      const double rr2 = (is_positive(b2) ? b2 : 0.0) * (ud * ud);
+      auto rres = [&]() {
+        const bool tiny = bits(rr2) < bits(1e-280);
+        const double r = sqrt(tiny ? (is_positive(b2) ? b2 : 0.0) : rr2);
+        return tiny ? r * fabs(ud) : r;
+      };
       const double bd = P.bd_tol * (amax + bmax);
       if (bits(b2) <= bits(bd * bd)) {  // bd is not negative; a negative b2 is the smaller one here too
         status = VS_DONE;  // invariant Krylov subspace: x_m is exact
@@ -647,14 +655,16 @@ __device__ __forceinline__ void finish_step_from(const StepParams& P, int j, int
       } else if (P.solve) {
         // linear solve: x_m = ||z|| V_m T_m^{-1} e_1 is the CG iterate, with
         // relative residual ||r_m|| / ||z|| = beta_m |e_m^T T_m^{-1} e_1|
-        const bool done = bits(rr2) <= bits(P.tol * P.tol);
-        if (done) status = VS_DONE;
-        else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
-        if (status != VS_RUNNING) err = sqrt(rr2);
+        if (bits(rr2) <= bits(P.tol * P.tol) || j + 1 >= P.m_max) {
+          const double r = rres();
+          if (r <= P.tol) status = VS_DONE;
+          else if (j + 1 >= P.m_max) status = GMRF_ERR_NOT_CONVERGED;
+          if (status != VS_RUNNING) err = r;
+        }
       } else if (bits(rr2) <= bits(P.tol * P.tol * (energy * theta)) || j + 1 >= P.m_max) {
         // est_lb = ||r_m|| / (||x_m|| theta^{1/2}), theta >= theta_min(T_m), is a lower bound of est
         need = 1;
-        pfac = sqrt(rr2) * rsqrt(energy);  // ||r_m|| / ||x_m||
+        pfac = rres() * rsqrt(energy);  // ||r_m|| / ||x_m||
         err = pfac * rsqrt(theta);
       }
     }
