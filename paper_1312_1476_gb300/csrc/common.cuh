@@ -368,6 +368,10 @@ __device__ __forceinline__ void vb_store4(__nv_bfloat16* p, float a, float b, fl
 // beta^2.  The determinants' recurrence takes one dependent FMA per row where the
 // pivots' takes a division; scale (a power of two near 1 / ||T_m||) and a power of two
 // every fourth row keep it in range.
+// Range: FP32 copies of T_m resolve eigenvalues down to about 1e-7 ||T_m||.  On spectra of
+// condition up to 1e8 this and the pivots' form answer alike; beyond, both answer by their
+// rounding, and pivots below about 10^-9.5 ||T_m|| in four consecutive rows underflow the
+// determinants to 0, which counts as an eigenvalue below sigma.
 __device__ __forceinline__ bool ritz_below(const float* __restrict__ af, const float* __restrict__ b2f, int m,
                                            float sigma, float scale) {
   float p1 = 1.f, p = (af[0] - sigma) * scale;
@@ -540,7 +544,7 @@ __device__ __forceinline__ double one_sum(double v) { return v; }
 // another's, both from beta_j^2; square roots of the estimate are taken only in a
 // step that may stop.  The state's fields are loaded ahead, one per lane, and
 // written one by one: a copy of the record costs the kernels this is inlined into
-// registers (spills in the 3-D step's item loop, 330 -> 344 us at 256^3, 8 vectors).
+// registers (spills in the 3-D step's item loop, 4 % of a step at 256^3, 8 vectors).
 // Only as many warps as there are partial sums take part in the sum.
 // With warp_sum3 and publish(), before and now: FP64 64 x 64 step 17.2 -> 11.7 us
 // (one vector; 12.7 with all of it in one warp), 93 -> 48 us (256 vectors); 512 x 512

@@ -31,10 +31,12 @@
 //
 // Measured on GB300 against the kernels this replaces (transforms both ways
 // along y on a transposed spectrum, one line per warp), FP32 MIRROR 1024 x 1024,
-// one vector: row-forward 9.3 -> 5.8 us, columns 11.2 -> 5.1, row-mid 14.2 -> 6.9,
-// row-last with the step's scalar tail 16.7 -> 12.4; 320 vectors of 512 x 512, 64
-// steps: 107 -> 65 ms; FP64 CIRCULANT 512 x 512 step 81 -> 42 us.  Error of
-// M^{-1/2} v against 64 bits at 128 x 128: 2.6e-7 -> 1.6e-7.
+// one vector, profiler times with a warm cache: row-forward 9.3 -> 6.0 us, columns 11.2 ->
+// 5.0, row-mid 14.2 -> 6.7, row-last with the step's scalar tail 16.7 -> 11.0; a step of an
+// untraced call 57 -> 30.3.  320 vectors of 512 x 512, about 58 steps: 108 -> 67 ms a call,
+// the passes of a step at 6.6 (row-forward), 5.3, 5.1 and 4.8 TB/s of their 17 arrays.  FP64
+// CIRCULANT 512 x 512 step 81 -> 42 us.  Error of M^{-1/2} v against 64 bits at 128 x 128:
+// 2.6e-7 -> 1.6e-7.
 #pragma once
 
 #include <cuda_runtime.h>

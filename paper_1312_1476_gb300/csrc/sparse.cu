@@ -16,8 +16,9 @@
 //     q_j = u - beta_{j-1} v_{j-1} -> W_out, the three dot products,
 // then alpha_j = v_j . q_j, beta_j = ||q_j - alpha_j v_j|| (a second pass over
 // the vectors in shared memory, exact also where A is close to the identity)
-// and the stopping rule (finish_step, common.cuh) in the same block.  Rows of one level depend only on rows of earlier levels, so
-// the threads of the block solve them in parallel with one barrier per level.
+// and the stopping rule (finish_step, common.cuh) in the same block.  Rows of one
+// merged level (tri_schedule.h) depend only on rows of earlier ones, so the threads
+// of the block solve them in parallel with one barrier per merged level.
 // Without F the step is u = Q v_j.
 #include <cuda_runtime.h>
 

@@ -21,12 +21,13 @@
 // straight from registers.  The z chunk depends on the grid alone, so a vector's
 // sums do not depend on its batch.
 //
-// Bound: instruction issue, about 45 per cell, on small grids the latency of the
-// planes one after another.  Measured against the register kernel this replaces,
-// whole sample calls to 1e-6: 61 x 75 x 90, 4 vectors, FP32 1208 -> 1028 us
-// (periodic 1946 -> 940), FP64 4725 -> 3410; 128 x 128 x 130, one vector, FP32 5286
-// -> 1268 (periodic 9781 -> 1200), FP64 35.5 -> 4.5 ms; 33 x 40 x 37, one vector, FP32
-// 636 -> 585, FP64 1197 -> 790.
+// Bound: instruction issue (61 x 75 x 90, 4 vectors: 59 % of the slots, 200 instructions per
+// cell with the chunks' halo planes, barriers next; 18.7 us a step), on smaller grids the
+// latency of the planes one after another.  Measured against the register kernel this
+// replaces, whole sample calls to 1e-6: 61 x 75 x 90, 4 vectors, FP32 1208 -> 1028 us
+// (periodic 1946 -> 940), FP64 4725 -> 3410; 128 x 128 x 130, one vector, FP32 5286 -> 1268
+// (periodic 9781 -> 1200), FP64 35.5 -> 4.5 ms; 33 x 40 x 37, one vector, FP32 636 -> 585, FP64
+// 1197 -> 790.
 #include <cuda_runtime.h>
 
 #include <algorithm>

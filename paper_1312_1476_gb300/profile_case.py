@@ -19,6 +19,9 @@ Cases:
                  larger than L2 that a counter capture can replay)
   stencil2d_1024 1024 x 1024 SPDE, zero-Neumann, no preconditioner, FP32 (the
                  streamed 2-D step), N vectors per launch
+  stencil2d_odd  701 x 999, 5-point, periodic, constant kappa^2, FP32 (strips of rows that are not aligned)
+  small_64       64 x 64, 5-point, periodic, constant kappa^2, FP64 (all steps of a vector in one cluster)
+  3d_odd         61 x 75 x 90 Dirichlet 7-point, kappa^2 i.i.d. U[0.01, 1], FP32 (flat ranges of cells)
   figure3_ichol  the Figure 3 matrix (31^2 G)^2 (n = 900, Section 5.2) in CSR,
                  incomplete-Cholesky factor (drop tolerance 1e-3, shift 1e-3),
                  FP64, N vectors per launch
@@ -47,6 +50,16 @@ def run(case: str, nsamples: int, steps: int, trace: bool = False) -> dict:
         prob = gmrf.Problem(shape, "neumann", "spde_squared", kappa2=k2)
     elif case in ("3d_256", "3d_128"):
         shape = (256, 256, 256) if case == "3d_256" else (128, 128, 128)
+        k2 = torch.from_numpy(inputs.kappa2_uniform_field(shape, seed=1)).cuda()
+        prob = gmrf.Problem(shape, "dirichlet", "shifted_laplacian", kappa2=k2)
+    elif case == "stencil2d_odd":
+        shape = (701, 999)
+        prob = gmrf.Problem(shape, "periodic", "shifted_laplacian", kappa2_const=0.1)
+    elif case == "small_64":
+        shape = (64, 64)
+        prob = gmrf.Problem(shape, "periodic", "shifted_laplacian", kappa2_const=0.1, precision="fp64")
+    elif case == "3d_odd":
+        shape = (61, 75, 90)
         k2 = torch.from_numpy(inputs.kappa2_uniform_field(shape, seed=1)).cuda()
         prob = gmrf.Problem(shape, "dirichlet", "shifted_laplacian", kappa2=k2)
     elif case == "figure3_ichol":
@@ -102,7 +115,7 @@ def run(case: str, nsamples: int, steps: int, trace: bool = False) -> dict:
 def main(argv=None):
     ap = argparse.ArgumentParser(description=__doc__.split("\n")[0])
     ap.add_argument("case", choices=["headline_1024", "batched_512", "3d_256", "3d_128", "stencil2d_1024",
-                                     "figure3_ichol"])
+                                     "stencil2d_odd", "small_64", "3d_odd", "figure3_ichol"])
     ap.add_argument("--nsamples", type=int, default=1)
     ap.add_argument("--steps", type=int, default=24)
     ap.add_argument("--trace", action="store_true", help="also report per-kernel-class times")
