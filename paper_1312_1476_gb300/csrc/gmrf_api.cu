@@ -176,13 +176,15 @@ int worst_status(const VecState* st, int nvec) {
   return worst;
 }
 
-// Runs the Lanczos iteration on the vectors already in W[0].  Returns a
-// gmrf code for launch failures only; per-vector outcomes are in st_host.
 // The grids whose steps one launch runs until its vectors stop; not where something
 // happens after each step (the two-pass accumulation, a timed launch).
 bool resident_steps(const gmrf_problem* p, const LanczosBufs& b) {
   return !p->sp && p->precond == GMRF_PREC_NONE && !b.Xacc && !trace_timing_enabled() &&
          stencil2d_resident_eligible(p->g, p->fp64, b.nvec);
+}
+
+void resident_ask(gmrf_problem* p, int nvec) {
+  if (!p->sp && p->precond == GMRF_PREC_NONE) stencil2d_resident_ask(p->g, p->fp64, nvec);
 }
 
 int launch_steps(gmrf_problem* p, const LanczosBufs& b, const StepParams& P, int c, cudaStream_t s) {
@@ -388,9 +390,12 @@ StepParams step_params(gmrf_problem* p, const LanczosBufs& b, double tol, int m_
   return P;
 }
 
+// Runs the Lanczos iteration on the vectors already in W[0].  Returns a
+// gmrf code for launch failures only; per-vector outcomes are in st_host.
 int run_lanczos(gmrf_problem* p, const LanczosBufs& b, double tol, int m_max, int check_every,
                 bool solve, bool init) {
   cudaStream_t s = p->ws;
+  resident_ask(p, b.nvec);
   if (init) CK(traced(KC_INIT, s, 1, [&] { return launch_lanczos_init(p->fp64, p->g.n, b, s); }));
   const StepParams P = step_params(p, b, tol, m_max, solve);
   const int c = std::min(check_every > 0 ? check_every : 16, m_max);
@@ -723,7 +728,6 @@ int gmrf_create(const gmrf_desc* d, void* stream, gmrf_problem** out) {
     delete p;
     return GMRF_ERR_CUDA;
   }
-  if (p->precond == GMRF_PREC_NONE) p->g.clusters = stencil2d_resident_fits(p->g, p->fp64);
   auto fail = [&](int code) {
     gmrf_destroy(p);
     return code;
@@ -1407,6 +1411,7 @@ int gmrf_autotune(gmrf_problem* p, int32_t nvec_max, gmrf_tuning* out) {
     P.tol = 1e-300;  // never met: every vector runs all timed steps
     P.bd_tol = p->fp64 ? 1e-13 : 1e-6;
     if (p->precond != GMRF_PREC_NONE) CKR(precond_prepare(p->pre, bw, s));
+    resident_ask(p, bw);
     CKR(capture_steps(p, b, P, kSteps));
     CK(cudaGraphLaunch(p->graph.exec, s));
     CK(cudaEventRecord(e0, s));

@@ -112,6 +112,7 @@ int ensure_lanczos(gmrf_problem* p, int nvec, int nslots, int m_max, bool need_t
 int batch_size(gmrf_problem* p, int want, int nslots, int m_max, bool need_tm, size_t extra_per_vec);
 int worst_status(const VecState* st, int nvec);
 int capture_steps(gmrf_problem* p, const LanczosBufs& b, const StepParams& P, int c);
+void resident_ask(gmrf_problem* p, int nvec);  // before the steps of nvec vectors are captured or launched
 int run_lanczos(gmrf_problem* p, const LanczosBufs& b, double tol, int m_max, int check_every, bool solve = false,
                 bool init = true);
 // The step parameters run_lanczos uses.

@@ -18,7 +18,7 @@ struct Grid {
   int bc;      // gmrf_bc
   int op;      // gmrf_op
   int zchunk = 0;  // 3-D FP32 stencil step: z planes per work item (0: chosen from the grid)
-  bool clusters = false;  // small 2-D grids: the device can place the clusters of stencil2d_resident.cu
+  int clusters = -1;  // small 2-D grids: whether the clusters of stencil2d_resident.cu can be placed (-1: not asked)
 };
 
 // Per-batch Lanczos buffers (all device pointers).  Element type T is float
@@ -63,9 +63,10 @@ int stencil_blocks_per_vector(const Grid& g);
 cudaError_t launch_stencil_step(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
                                 const LanczosBufs& b, const StepParams& P, cudaStream_t s, int nsteps = 1);
 bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec);
-// For Grid::clusters, once per problem and outside any capture: whether the grid is one of
-// them and a cluster of its size fits the current context, which may be limited to a few SMs.
-bool stencil2d_resident_fits(const Grid& g, bool fp64);
+// Asks for Grid::clusters on the first use of a problem with so few vectors, outside any
+// capture: whether a cluster of the grid's size fits the current context, which may be
+// limited to a few SMs.
+void stencil2d_resident_ask(Grid& g, bool fp64, int nvec);
 // y = Q v for nvec vectors (no Lanczos bookkeeping).
 cudaError_t launch_stencil_apply(const Grid& g, bool fp64, const void* kappa2, double kappa2_const,
                                  const void* v, void* y, int nvec, cudaStream_t s, double scale = 1.0);

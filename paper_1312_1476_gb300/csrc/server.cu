@@ -232,6 +232,7 @@ int step_body(gmrf_server* sv, int32_t* active) {
     const StepParams P = step_params(p, bp, sv->o.tol, sv->o.m_max, false);
     const int c = std::min(sv->o.check_every > 0 ? sv->o.check_every : 16, sv->o.m_max);
     if (p->precond != GMRF_PREC_NONE && !p->sp) CKR(precond_prepare(p->pre, hw8, s));
+    resident_ask(p, hw8);
     CKR(capture_steps(p, bp, P, c));
     CK(cudaGraphLaunch(p->graph.exec, s));
     trace_replayed(&p->graph.tr, c * p->graph.kernels_per_step);

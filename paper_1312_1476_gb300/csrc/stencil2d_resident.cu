@@ -309,10 +309,10 @@ static bool takes(const Grid& g, bool fp64, int nvec) {
   if (tiles <= kMaxCluster) return all <= (fp64 ? 5 : 2) * 152;
   return tiles <= (fp64 ? 3 * kMaxCluster : kMaxTiles) && all <= (fp64 ? 152 : 256);
 }
-bool stencil2d_resident_fits(const Grid& g, bool fp64) {
-  return takes(g, fp64, 1) && (fp64 ? fits<double>(g) : fits<float>(g));
+void stencil2d_resident_ask(Grid& g, bool fp64, int nvec) {
+  if (g.clusters < 0 && takes(g, fp64, nvec)) g.clusters = (fp64 ? fits<double>(g) : fits<float>(g)) ? 1 : 0;
 }
-bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec) { return g.clusters && takes(g, fp64, nvec); }
+bool stencil2d_resident_eligible(const Grid& g, bool fp64, int nvec) { return g.clusters > 0 && takes(g, fp64, nvec); }
 
 template <typename T>
 cudaError_t launch_stencil2d_resident(const Grid& g, const StencilArgs<T>& a, int nvec, int nsteps, cudaStream_t s) {
