@@ -91,8 +91,9 @@ __device__ __forceinline__ void ldk_s(const float* p, float (&o)[VX]) {
 // rows may start anywhere and the last strip ends inside: the copies move single
 // elements, lane after lane, the rows of v_j and q_j go out the same way from
 // shared memory, and cells outside the grid are kept out of g and of the sums;
-// the arithmetic between is the same.  Measured on 701 x 999, 16 vectors, 5-point,
-// against the tile kernel of lanczos_stencil.cu: 298 -> 61 us a step.
+// the arithmetic between is the same.  Measured on 701 x 999, 16 vectors, 5-point, 67
+// steps, against the tile kernel of lanczos_stencil.cu: 24.0 -> 4.87 ms a call (68 us a
+// step, 26 of them its bytes; bound by issue, 161 instructions per cell).
 template <typename T, int OP, int BC, bool STEP, bool AL>
 __global__ void __launch_bounds__(SNT) k_stencil2d_strip(StencilArgs<T> a, int ychunk) {
   constexpr int VX = strip_vx<T>(), BX = strip_bx<T>(), PW = BX + 2 * VX;
